@@ -80,6 +80,15 @@ __device__ __forceinline__ float sigmoid_fast(float g) {
   return r;
 }
 
+// ---- routing weights as matrix fragments --------------------------------------------------
+// The bf16 hi / lo parts of w [S, E] in the order the merge's matrix instructions hold their A operand: for every
+// group of 16 segments and 16 experts, hi then lo, 32 lanes of 16 bytes.  Offset (in bf16) of the hi part of w[s, e];
+// the lo part lies 256 further.  ktiles = ceil(E / 16).
+__host__ __device__ __forceinline__ size_t w_frag_offset(size_t s, int e, int ktiles) {
+  const int row = (int)(s & 15), col = e & 15;
+  return (((s >> 4) * ktiles + (e >> 4)) * 64 + (row & 7) * 4 + ((col & 7) >> 1)) * 8 + ((row >> 3) + 2 * (col >> 3)) * 2 + (col & 1);
+}
+
 // ---- device status word -----------------------------------------------------------------
 // Kernels with bounded waits OR a non-zero code into this word when a wait gives up.
 enum : uint32_t { STATUS_OK = 0, STATUS_TIMEOUT_TMA = 1, STATUS_TIMEOUT_MMA = 2, STATUS_TIMEOUT_EPI = 4,

@@ -106,7 +106,7 @@ static Layout make_layout(const lory_dims& D) {
   Lo.k_chunk = 8192;
   int simt_slabs = 3 * (int)ceil_div((long)P1, Lo.k_chunk);
   Lo.n_slabs = use_tc(D) ? tc_dw_slabs(D) : simt_slabs;
-  Lo.dw_partial = take((size_t)Lo.n_slabs * S * D.E * 4);
+  Lo.dw_partial = take((size_t)(use_tc(D) ? tc_dw_slabs_max(D) : simt_slabs) * S * D.E * 4);
   Lo.dw = take(S * D.E * 4);
   Lo.dz = take(S * D.E * 4);
   Lo.dh_bar = take(S * D.d * 4);
@@ -308,7 +308,7 @@ static int forward_impl(const lory_dims& D, const Layout& Lo, const T* x, const 
     RouteExtra extra;
     extra.w_copy = route_w;
     if (D.dtype == LORY_BF16 && use_tc(D)) {
-      tc_split_tables(D, Lo, ws, &extra.hi, &extra.lo, &extra.comb, &extra.Epad);
+      tc_split_tables(D, Lo, ws, &extra.hi, &extra.lo, &extra.comb, &extra.Epad, &extra.frag);
       w_is_split = true;
     }
     LORY_TRY(launch_pool_router<T>(x, w_r, (float*)(ws + Lo.h_bar), (float*)(ws + Lo.p), route_p, w, D.B, N, D.T,

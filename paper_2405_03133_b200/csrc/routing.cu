@@ -103,6 +103,16 @@ __device__ __forceinline__ void write_weight_row(const float* p_sm, size_t row, 
       ex.lo[row * ex.Epad + e] = __float2bfloat16_rn(v - __bfloat162float(h));
     }
   }
+  if (ex.frag) {
+    const int kt = (E + 15) >> 4;
+    for (int e = lane; e < kt * 16; e += 32) {
+      const float v = e < E ? p_sm[e] : 0.f;
+      const bf16 h = __float2bfloat16_rn(v);
+      bf16* dst = ex.frag + w_frag_offset(row, e, kt);
+      dst[0] = h;
+      dst[256] = __float2bfloat16_rn(v - __bfloat162float(h));
+    }
+  }
   if (ex.comb) {
     // [hi | lo | hi | hi | lo | lo], 32 columns each
     for (int c = lane; c < 192; c += 32) {

@@ -9,13 +9,15 @@ namespace lory {
 // prefix != 0: prefix routing (every segment of a sequence uses its first segment's p).
 // Optional extra outputs of the routing step, written by the router kernel itself:
 // a second copy of the routing weights (the caller's route_w), and the bf16 hi + lo tables of the weights that
-// the tensor-core merge reads: hi, lo [S, Epad]; comb [S, 192] = [hi | lo | hi | hi | lo | lo] in groups of 32 columns (E <= 32 only).
+// the tensor-core merge reads: hi, lo [S, Epad]; comb [S, 192] = [hi | lo | hi | hi | lo | lo] in groups of 32 columns (E <= 32 only);
+// frag: the same in the merge's fragment order (w_frag_offset).
 struct RouteExtra {
   float* w_copy = nullptr;
   bf16* hi = nullptr;
   bf16* lo = nullptr;
   bf16* comb = nullptr;
   int Epad = 0;
+  bf16* frag = nullptr;
 };
 template <typename T>
 int launch_pool_router(const T* x, const T* w_r, float* h_bar, float* p_ws, float* route_p, float* w_out,

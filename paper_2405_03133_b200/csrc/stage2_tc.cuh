@@ -12,13 +12,13 @@
 // hi-weighted sums in accumulator rows 0..63 and lo-weighted sums in rows 64..127; the epilogue adds
 // the two halves.  With E <= 32 one 64-wide table holds hi in columns 0..31 and lo in 32..63 and is placed
 // in shared memory twice, so that all four epilogue warps have work: two per 64-column half of the tile.  The dw accumulator stays in TMEM for the whole kernel.
-// With E <= 32 and at most 64 segments (p.fast) the first product runs as two MMAs per 16 segments, [hi|hi] and
-// [lo|lo] tables into ONE accumulator: every 32-lane quarter then holds the finished sums of all experts, and the
-// epilogue warps take whole tiles in turn (two per accumulator, one 64-column half each) without exchanging
-// anything (d = 2048, f = 5504: E = 32, S = 16: 1.52 -> 1.17 ms; S = 64: 1.95 -> 1.64 ms; E = 16, S = 64: 1.65 -> 1.54 ms;
-// at S = 128 the doubled MMA count costs more than it saves, so the arrangement above stays there).
-// With 17..64 segments a tile of this arrangement is 192 columns wide (three blocks; block b of a CTA's i-th tile
-// goes to epilogue warp (3 i + b) mod 4): a third fewer MMAs of the first product per byte.
+// Used where the streaming adjoint (stream_tc.cuh) cannot keep its dw sums in registers.  With E <= 32 and at most 64
+// segments (p.fast) the first product runs as two MMAs per 16 segments, [hi|hi] and [lo|lo] tables into ONE accumulator:
+// every 32-lane quarter then holds the finished sums of all experts, and the epilogue warps take whole tiles in turn (one
+// 64-column block each) without exchanging anything (d = 2048, f = 5504, E = 32, S = 64: 1.95 -> 1.64 ms; at S = 128 the
+// doubled MMA count costs more than it saves, so the arrangement above stays there).  A tile of this arrangement is 192
+// columns wide (three blocks; block b of a CTA's i-th tile goes to epilogue warp (3 i + b) mod 4): a third fewer MMAs of
+// the first product per byte.
 // Roles: warp 0 TMA, warp 1 issues the first product and owns TMEM, warps 2..5 epilogue, warp 6 issues the second
 // product.  Two issuing threads because with few segments a tile is small (24 KB at S = 64) and the instruction
 // stream of ONE thread issuing both products (12 MMAs with their descriptors, 2 commits, 2 waits) was what a tile
@@ -47,8 +47,7 @@ struct Stage2Maps {
 struct Stage2Params {
   int S, E, Epad16, s_tiles;  // S: segments of this launch (at most 256); s_tiles = ceil(S / 128)
   int seg_base, S_total;      // first segment of this launch; all segments (row count of a dw slab)
-  int rpt_shift;    // 0: a tile is ncb * 64 columns of one row; 1: 64 columns of two neighbouring rows
-  int ncb;          // 64-column blocks of a tile: 2, or 3 on the fast path with 33..64 segments (fewer MMAs per byte)
+  int ncb;          // 64-column blocks of a tile (of one row): 2, or 3 on the fast path (fewer MMAs per byte)
   int ctiles[3];    // column tiles per row
   uint32_t cmagic[3];  // ceil(2^32 / ctiles), 0 for ctiles == 1: n / ctiles == __umulhi(n, cmagic) for every tile index n
   int tile_end[3];  // exclusive prefix sums of (rows rounded up to 64) * ctiles
@@ -98,11 +97,8 @@ stage2_kernel(const __grid_constant__ Stage2Maps maps, const Stage2Params p) {
     const int local = tile - (k == 0 ? 0 : p.tile_end[k - 1]);
     // local / ctiles[k] without the division (a single tile per row has no 32-bit reciprocal: magic 0)
     r = p.cmagic[k] ? (int)__umulhi((uint32_t)local, p.cmagic[k]) : local;
-    c0 = (local - r * p.ctiles[k]) * (p.rpt_shift ? 64 : NCB * 64);
-    r <<= p.rpt_shift;
+    c0 = (local - r * p.ctiles[k]) * (NCB * 64);
   };
-  // the two 64-column halves of a tile: columns c0 and c0 + 64 of row r, or (two-row tiles) column c0 of rows r, r + 1
-  const int half_col = p.rpt_shift ? 0 : 64, half_row = p.rpt_shift ? 1 : 0;
   const uint32_t ACC_COLS = (uint32_t)NCB * 64u;   // TMEM columns of one per-tile accumulator
 
   // debug build: a decoded tile against the padded tile grid of its matrix
@@ -110,7 +106,7 @@ stage2_kernel(const __grid_constant__ Stage2Maps maps, const Stage2Params p) {
     if (!dbg::kOn) return true;
     if (k < 0 || k > 2) return false;
     const int tiles_k = p.tile_end[k] - (k ? p.tile_end[k - 1] : 0);
-    return dbg::coord_ok(r, (tiles_k / p.ctiles[k]) << p.rpt_shift) && dbg::inner_ok(c0, p.ctiles[k] * (p.rpt_shift ? 64 : NCB * 64));
+    return dbg::coord_ok(r, tiles_k / p.ctiles[k]) && dbg::inner_ok(c0, p.ctiles[k] * (NCB * 64));
   };
 
   if (threadIdx.x == 0) {
@@ -199,16 +195,10 @@ stage2_kernel(const __grid_constant__ Stage2Maps maps, const Stage2Params p) {
           ptx::mbar_expect_tx(&full_bar[s], tx);
           issued |= 1u << s;
           last_parity = (last_parity & ~(1u << s)) | (ph << s);
-          // (col in block, row in block, segment, col block, row block): two col blocks, 128 segments
-          if (p.rpt_shift) {  // two boxes of one column block each (rows r, r + 1)
-            ptx::tma_load_5d(sD, &maps.dwbar[k], &full_bar[s], 0, r & 63, p.seg_base + st * 128, c0 >> 6, r >> 6);
-            ptx::tma_load_5d(sD + p.cb_stride, &maps.dwbar[k], &full_bar[s], 0, (r & 63) + 1, p.seg_base + st * 128,
-                             c0 >> 6, r >> 6);
-          } else {            // one box of two column blocks
-            ptx::tma_load_5d(sD, &maps.dwbar[k], &full_bar[s], 0, r & 63, p.seg_base + st * 128, c0 >> 6, r >> 6);
-          }
+          // (col in block, row in block, segment, col block, row block): one box of NCB column blocks
+          ptx::tma_load_5d(sD, &maps.dwbar[k], &full_bar[s], 0, r & 63, p.seg_base + st * 128, c0 >> 6, r >> 6);
           for (int j = 0; j < NCB; ++j)
-            ptx::tma_load_3d(sT + j * p.Epad16 * 128, &maps.theta[k], &full_bar[s], c0 + j * half_col, 0, r + j * half_row);
+            ptx::tma_load_3d(sT + j * p.Epad16 * 128, &maps.theta[k], &full_bar[s], c0 + j * 64, 0, r);
         }
       }
       if (abort_flag) {
@@ -344,7 +334,7 @@ stage2_kernel(const __grid_constant__ Stage2Maps maps, const Stage2Params p) {
         }
         uint32_t r[64];
         ptx::tmem_ld_32x64(taddr, r);
-        const int col0 = c0 + half * half_col, rowc = row + half * half_row;
+        const int col0 = c0 + half * 64, rowc = row;
         uint4 old[8];
         if (ACC) {  // gradient accumulation: this lane's 64 old values (expert `lane`), zero where the tile leaves the tensor
           const bool row_ok = lane < p.E && rowc < p.rows[k];
@@ -431,7 +421,7 @@ stage2_kernel(const __grid_constant__ Stage2Maps maps, const Stage2Params p) {
           // the tile leaves the tensor
           uint4 old[8];
           if (ACC) {
-            const int e = e0 + lane, col0 = c0 + c * half_col, rowc = row + c * half_row;
+            const int e = e0 + lane, col0 = c0 + c * 64, rowc = row;
             const bool row_ok = e < p.E && rowc < p.rows[k];
             const __nv_bfloat16* src = p.acc_base[k] + (size_t)e * p.e_stride[k] + (size_t)rowc * p.row_stride[k] + col0;
 #pragma unroll
@@ -464,7 +454,7 @@ stage2_kernel(const __grid_constant__ Stage2Maps maps, const Stage2Params p) {
             ptx::tc_fence_before_sync();
             ptx::mbar_arrive(&tmem_empty_bar[acc]);
           }
-          warp_stage_and_store(wsg, &maps.out[k], c0 + c * half_col, e0, row + c * half_row, lane, w);
+          warp_stage_and_store(wsg, &maps.out[k], c0 + c * 64, e0, row, lane, w);
         }
       }
     }

@@ -17,8 +17,8 @@
 #include <stdlib.h>
 
 #include "gemm_tc.cuh"
-#include "merge_tc.cuh"
 #include "stage2_tc.cuh"
+#include "stream_tc.cuh"
 #include "wgrad_tc.cuh"
 
 namespace lory {
@@ -235,8 +235,8 @@ static int e_pad16(const lory_dims& D) { return (D.E + 15) / 16 * 16; }
 // of 32 columns, [hi | lo | hi | hi | lo | lo] (zero where e >= E): the merge adjoint reads columns 0..63 or
 // 64..191 of it; the grid then covers S x 192.
 __global__ void split_w_kernel(const float* __restrict__ w, bf16* __restrict__ hi, bf16* __restrict__ lo,
-                               bf16* __restrict__ comb, int S, int E, int Epad) {
-  const int width = E <= 32 ? 192 : Epad;
+                               bf16* __restrict__ comb, bf16* __restrict__ frag, int S, int E, int Epad) {
+  const int kt = (E + 15) >> 4, width = E <= 32 ? 192 : kt * 16;
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= S * width) return;
   const int s = i / width, c = i - s * width;
@@ -247,15 +247,20 @@ __global__ void split_w_kernel(const float* __restrict__ w, bf16* __restrict__ h
   if (E <= 32) {
     const int part = c >> 5;
     comb[i] = (part == 0 || part == 2 || part == 3) ? h : l;
-    if (c >= Epad) return;
   }
+  if (c < kt * 16) {
+    bf16* dst = frag + w_frag_offset(s, c, kt);
+    dst[0] = h;
+    dst[256] = l;
+  }
+  if (c >= Epad) return;
   hi[(size_t)s * Epad + e] = h;
   lo[(size_t)s * Epad + e] = l;
 }
 
 size_t tc_w_split_bytes(const lory_dims& D) {
   const size_t S = (size_t)D.B * (D.L / D.T);
-  return 2 * align_up(S * e_pad(D) * 2, 256) + align_up(S * 192 * 2, 256);
+  return 2 * align_up(S * e_pad(D) * 2, 256) + align_up(S * 192 * 2, 256) + align_up((S + 15) / 16 * 16 * e_pad16(D) * 4, 256);
 }
 
 // The merge and merge-adjoint kernels keep the routing weights of the segments they work on resident in shared
@@ -270,12 +275,6 @@ size_t tc_blocked_elems(const lory_dims& D, int R, int C) {
   return (size_t)((R + 63) / 64) * ((C + 63) / 64) * S * 4096;
 }
 
-// Two-row tiles (64 columns of rows r, r + 1) pay off only with very few segments, where the expert traffic dominates
-// (S = 16: 1.67 -> 1.56 ms at d = 2048, f = 5504, E = 32); at S >= 64 they measure the same as 128 columns of one row,
-// and at S = 32 the three-block tiles below are better (1.42 -> 1.34 ms).
-static int stage2_rpt_shift(const lory_dims& D) {
-  return D.B * (D.L / D.T) <= 16 ? 1 : 0;
-}
 // One of the (up to three) parameter rectangles a launch of the merge adjoint covers: a whole expert matrix, or a
 // sub-rectangle of one whose per-segment gradients sit in a buffer of their own.  R == 0: not part of the launch.
 struct AdjPiece {
@@ -285,21 +284,17 @@ struct AdjPiece {
   int R, C;
   uint64_t e_stride, row_stride;  // elements between experts / rows of W_k and dW_k
 };
-// Tiles of three 64-column blocks instead of two where both weight halves go through the tensor core (E <= 32,
-// 17..64 segments): the first product then needs its MMAs once per 192 columns instead of once per 128, and the MMA
-// count is what a tile waits for there (d = 2048, f = 5504: E = 16, S = 64: 1.54 -> 1.34 ms; E = 32, S = 64: 1.64 -> 1.58;
-// S = 32: 1.42 -> 1.34).  Four blocks would not fit TMEM beside the double buffering.
-static int stage2_ncb(const lory_dims& D) {
-  const int S = D.B * (D.L / D.T);
-  return (D.E <= 32 && S > 16 && S <= 64) ? 3 : 2;
-}
+// Tiles of three 64-column blocks instead of two where both weight halves go through the tensor core (E <= 32, at most
+// 64 segments): the first product then needs its MMAs once per 192 columns instead of once per 128, and the MMA count is
+// what a tile waits for there (d = 2048, f = 5504, E = 32, S = 64: 1.64 -> 1.58 ms).  Four blocks would not fit TMEM beside
+// the double buffering.
+static int stage2_ncb(const lory_dims& D) { return (D.E <= 32 && D.B * (D.L / D.T) <= 64) ? 3 : 2; }
 static void stage2_tiles(const lory_dims& D, const int R[3], const int C[3], int ctiles[3], int tile_end[3]) {
-  const int rsh = stage2_rpt_shift(D);
-  const int width = rsh ? 64 : stage2_ncb(D) * 64;   // columns per tile
+  const int width = stage2_ncb(D) * 64;   // columns per tile
   int acc = 0;
   for (int k = 0; k < 3; ++k) {
     ctiles[k] = C[k] > 0 ? (C[k] + width - 1) / width : 1;
-    acc += (((R[k] + 63) / 64 * 64) >> rsh) * ctiles[k];  // whole row blocks: the rows past R[k] read zeros and store nothing
+    acc += (R[k] + 63) / 64 * 64 * ctiles[k];  // whole row blocks: the rows past R[k] read zeros and store nothing
     tile_end[k] = acc;
   }
 }
@@ -310,7 +305,51 @@ static int stage2_grid(const lory_dims& D) {
   return te[2] < sm_count() ? te[2] : sm_count();
 }
 
-int tc_dw_slabs(const lory_dims& D) { return stage2_grid(D); }
+// Where the adjoint of the merge runs as a streaming kernel (stream_tc.cuh): as long as a warp can keep the dw sums of
+// all segments and experts (and, for 17..32 experts, its pieces' rows in flight) beside its working set.  Measured at
+// d = 1024, f = 2752 against the tcgen05 kernel: E = 16, S = 64: 306 -> 271 us; E = 32, S = 48: 365 -> 326 us, but S = 64:
+// 381 -> 475 us; E = 48, S = 32: 617 -> 398 us.
+static bool adjoint_streams(const lory_dims& D) {
+  const int st = (D.B * (D.L / D.T) + 15) / 16, et = (D.E + 15) / 16;
+  return st <= (et == 1 ? 4 : (et == 2 ? 3 : 2));
+}
+template <int ST, int ET>
+struct StreamShape {
+  static constexpr int S16 = ST, E16 = ET;
+};
+// calls f with the template shape of the streaming adjoint for these dims (adjoint_streams holds)
+template <typename F>
+static int for_stream_shape(const lory_dims& D, F f) {
+  const int st = (D.B * (D.L / D.T) + 15) / 16, et = (D.E + 15) / 16;
+  switch (et * 8 + st) {
+    case 8 + 1: return f(StreamShape<1, 1>());
+    case 8 + 2: return f(StreamShape<2, 1>());
+    case 8 + 3: return f(StreamShape<3, 1>());
+    case 8 + 4: return f(StreamShape<4, 1>());
+    case 16 + 1: return f(StreamShape<1, 2>());
+    case 16 + 2: return f(StreamShape<2, 2>());
+    case 16 + 3: return f(StreamShape<3, 2>());
+    case 24 + 1: return f(StreamShape<1, 3>());
+    case 24 + 2: return f(StreamShape<2, 3>());
+    case 32 + 1: return f(StreamShape<1, 4>());
+    case 32 + 2: return f(StreamShape<2, 4>());
+    default: return LORY_ERR_SHAPE;
+  }
+}
+static int adjoint_stream_ctas(const lory_dims& D, bool acc) {
+  return for_stream_shape(D, [&](auto shape) {
+    using S = decltype(shape);
+    return acc ? AdjointStream<S::S16, S::E16, true>::CTAS : AdjointStream<S::S16, S::E16, false>::CTAS;
+  }) * sm_count();
+}
+int tc_dw_slabs(const lory_dims& D) {
+  return adjoint_streams(D) ? adjoint_stream_ctas(D, (D.flags & LORY_FLAG_ACCUMULATE_GRADS) != 0) : stage2_grid(D);
+}
+int tc_dw_slabs_max(const lory_dims& D) {
+  if (!adjoint_streams(D)) return stage2_grid(D);
+  const int a = adjoint_stream_ctas(D, true), b = adjoint_stream_ctas(D, false);
+  return a > b ? a : b;
+}
 
 // ---------------------------------------------------------------------------------------
 // Chunked adjoint (LORY_FLAG_CHUNKED_ADJOINT): the per-segment weight gradients of one rectangle of one expert
@@ -368,7 +407,7 @@ static bool use_pairs(int rows) { return rows % 256 == 0; }
 struct WsPtrs {
   uint32_t* status;
   const float* w;
-  bf16 *w_hi, *w_lo, *w_comb, *wbar1, *wbar3, *wbar2, *G, *U, *H, *dG, *dU, *dwbar1, *dwbar3, *dwbar2;
+  bf16 *w_hi, *w_lo, *w_comb, *w_frag, *wbar1, *wbar3, *wbar2, *G, *U, *H, *dG, *dU, *dwbar1, *dwbar3, *dwbar2;
   float* dw_partial;
 };
 static WsPtrs ws_ptrs(const lory_dims& D, const Layout& Lo, char* ws) {
@@ -379,6 +418,7 @@ static WsPtrs ws_ptrs(const lory_dims& D, const Layout& Lo, char* ws) {
   q.w_hi = (bf16*)(ws + Lo.w_split);
   q.w_lo = (bf16*)(ws + Lo.w_split + align_up((size_t)S * e_pad(D) * 2, 256));
   q.w_comb = (bf16*)(ws + Lo.w_split + 2 * align_up((size_t)S * e_pad(D) * 2, 256));
+  q.w_frag = (bf16*)((char*)q.w_comb + align_up((size_t)S * 192 * 2, 256));
   q.wbar1 = (bf16*)(ws + Lo.wbar1); q.wbar3 = (bf16*)(ws + Lo.wbar3); q.wbar2 = (bf16*)(ws + Lo.wbar2);
   q.G = (bf16*)(ws + Lo.G); q.U = (bf16*)(ws + Lo.U); q.H = (bf16*)(ws + Lo.H);
   q.dG = (bf16*)(ws + Lo.dG); q.dU = (bf16*)(ws + Lo.dU);
@@ -387,56 +427,95 @@ static WsPtrs ws_ptrs(const lory_dims& D, const Layout& Lo, char* ws) {
   return q;
 }
 
+// The streaming kernels move 16-byte vectors: the caller's expert tensors have to start on such a boundary (the tensor
+// maps of the other kernels ask for the same).
+static int check_vector_aligned(const void* const* ptrs, int n) {
+  for (int i = 0; i < n; ++i) {
+    if ((uintptr_t)ptrs[i] & 15) {
+      CallState& s = call_state();
+      snprintf(s.cuda_error, sizeof(s.cuda_error), "an expert tensor does not start on a 16-byte boundary");
+      return LORY_ERR_CUDA;
+    }
+  }
+  return LORY_OK;
+}
+
+template <int KT, int U, int NW>
+static int launch_merge_t(const StreamMergeParams& p, cudaStream_t st) {
+  ProfScope ps("merge", st);
+  merge_stream_kernel<KT, U, NW><<<(unsigned)ceil_div(p.piece_end[2], NW * U), 32 * NW, 0, st>>>(p);
+  LORY_AFTER_LAUNCH();
+  return LORY_OK;
+}
 // Wbar_k (blocked) = (w_hi + w_lo) . W_k for the three matrices in one launch      (Eq. 2)
 static int launch_merge(const lory_dims& D, const WsPtrs& q, const bf16* const src[3], bf16* const dst[3],
                         cudaStream_t st) {
-  const int S = D.B * (D.L / D.T), E = D.E, Ep = e_pad(D);
   const int R[3] = {D.f, D.f, D.d}, C[3] = {D.d, D.d, D.f};
-  MergeMaps maps;
-  MergeParams p = {};
-  const int S_launch = S < 256 ? S : 256;  // the routing weights of at most 256 segments stay in shared memory
-  p.S = S_launch; p.E = E; p.Epad16 = e_pad16(D); p.s_tiles = (S_launch + 127) / 128; p.status = q.status;
-  p.dup = S <= 32 ? 2 : (S <= 64 ? 1 : 0);
-  // Tiles of 4 rows x 64 columns: a segment's four 128-byte output pieces of one tile are neighbours in its 64 x 64
-  // block (512 contiguous bytes).  Measured against 1 x 256 and 2 x 128: C3 0.546 / 0.520 / 0.524 ms (1, 2, 4 rows),
-  // C4 1.064 / 1.036 / 0.996 ms.
-  p.rpt_shift = 2;
-  const uint32_t w_box = p.dup == 2 ? 32u : (p.dup ? 64u : 128u);
-  LORY_TRY(make_map(&maps.w_hi, q.w_hi, Ep, S, 1, Ep, 0, w_box));
-  LORY_TRY(make_map(&maps.w_lo, q.w_lo, Ep, S, 1, Ep, 0, w_box));
-  int acc = 0;
+  LORY_TRY(check_vector_aligned((const void* const*)src, 3));
+  StreamMergeParams p = {};
+  unsigned long pieces = 0;
   for (int k = 0; k < 3; ++k) {
-    LORY_TRY(make_expert_map(&maps.theta[k], src[k], R[k], C[k], E, p.Epad16));
-    LORY_TRY(make_blocked_map(&maps.out[k], dst[k], R[k], C[k], S, 1, S < 32 ? (uint32_t)S : 32u, 1, 1));  // no box rows past the segments
-    p.ctiles[k] = (C[k] + (256 >> p.rpt_shift) - 1) / (256 >> p.rpt_shift);
-    acc += (((R[k] + 63) / 64 * 64) >> p.rpt_shift) * p.ctiles[k];  // padded rows are written too (as zeros)
-    p.tile_end[k] = acc;
+    p.src[k] = src[k]; p.dst[k] = dst[k]; p.R[k] = R[k]; p.C[k] = C[k]; p.Cb[k] = (C[k] + 63) / 64;
+    pieces += (unsigned long)((R[k] + 63) / 64 * 64) * p.Cb[k];
+    p.piece_end[k] = (unsigned)pieces;
   }
-  p.stage_bytes = 4 * p.Epad16 * 128;
-  const int fixed = p.s_tiles * 32768 + 32768 + 1024;
-  p.stages = (kMaxSmem - fixed) / p.stage_bytes;
-  if (p.stages > 8) p.stages = 8;
-  if (p.stages < 2) return LORY_ERR_SHAPE;
-  const int smem = fixed + p.stages * p.stage_bytes;
-  static bool attr_set[kMaxDevices];
-  LORY_TRY(allow_dynamic_smem(merge_kernel, kMaxSmem, attr_set));
-  const int grid = p.tile_end[2] < sm_count() ? p.tile_end[2] : sm_count();
-  // one launch per 256 segments (each re-reads the experts once: the same ratio as one launch at S = 256)
-  for (int base = 0; base < S; base += 256) {
-    p.seg_base = base;
-    p.S = S - base < 256 ? S - base : 256;
-    p.s_tiles = (p.S + 127) / 128;
-    ProfScope ps("merge", st);
-    merge_kernel<<<grid, 192, smem, st>>>(maps, p);
-    LORY_AFTER_LAUNCH();
+  if (pieces > 0x7fffffffUL) return LORY_ERR_SHAPE;
+  p.w_frag = (const uint4*)q.w_frag; p.S = D.B * (D.L / D.T); p.E = D.E;
+  // Loads in flight per warp: 8 vectors per lane with up to 32 experts (two pieces of 16 experts or one of 32; two of 32
+  // cost occupancy: 1.13 instead of 1.02 ms at S = 64, d = 2048, f = 5504), one piece with more.
+  switch ((D.E + 15) / 16) {
+    case 1: return launch_merge_t<1, 2, 2>(p, st);
+    case 2: return launch_merge_t<2, 1, 2>(p, st);
+    case 3: return launch_merge_t<3, 1, 2>(p, st);
+    default: return launch_merge_t<4, 1, 4>(p, st);
   }
-  return LORY_OK;
+}
+
+static int launch_adjoint_stream(const lory_dims& D, const WsPtrs& q, const AdjPiece pc[3], bool slab_add, cudaStream_t st) {
+  StreamAdjointParams p = {};
+  unsigned long pieces = 0;
+  for (int k = 0; k < 3; ++k) {
+    const AdjPiece& a = pc[k];
+    if (a.R > 0) {
+      const void* const ptrs[2] = {a.wsrc, a.ddst};
+      LORY_TRY(check_vector_aligned(ptrs, 2));
+      p.dsrc[k] = a.dsrc; p.wsrc[k] = a.wsrc; p.ddst[k] = a.ddst;
+      p.R[k] = a.R; p.C[k] = a.C; p.Cb[k] = (a.C + 63) / 64;
+      p.e_stride[k] = (long)a.e_stride; p.row_stride[k] = (long)a.row_stride;
+      pieces += (unsigned long)a.R * p.Cb[k];
+    }
+    p.piece_end[k] = (unsigned)pieces;
+  }
+  if (pieces == 0) return LORY_OK;
+  if (pieces > 0x7fffffffUL) return LORY_ERR_SHAPE;
+  p.w = q.w; p.S = D.B * (D.L / D.T); p.E = D.E; p.slab_add = slab_add ? 1 : 0; p.dw_partial = q.dw_partial;
+  const bool acc = (D.flags & LORY_FLAG_ACCUMULATE_GRADS) != 0;
+  const int ctas = tc_dw_slabs(D);
+  return for_stream_shape(D, [&](auto shape) -> int {
+    using S = decltype(shape);
+    auto launch = [&](auto kern, auto cfg, bool (&done)[kMaxDevices]) -> int {
+      using A = decltype(cfg);
+      // Two stages once the pieces on their way then hold 70 KB per SM (read and written rows counted), else three.
+      // More is worse, not only useless: E = 16, S = 16, d = 2048: 548 us with two stages, 618 with three; E = 12, S = 12:
+      // 459 with two, 436 with three.
+      p.stages = A::STG >= 3 && A::CTAS * A::NW * (p.S + 2 * p.E) * 128 < 70 * 1024 ? 3 : 2;
+      LORY_TRY(allow_dynamic_smem(kern, A::SMEM, done));
+      ProfScope ps("stage2", st);
+      kern<<<ctas, 32 * A::NW, A::SMEM, st>>>(p);
+      LORY_AFTER_LAUNCH();
+      return LORY_OK;
+    };
+    static bool done[2][kMaxDevices];
+    if (acc) return launch(adjoint_stream_kernel<S::S16, S::E16, true>, AdjointStream<S::S16, S::E16, true>(), done[1]);
+    return launch(adjoint_stream_kernel<S::S16, S::E16, false>, AdjointStream<S::S16, S::E16, false>(), done[0]);
+  });
 }
 
 // dW_k = w^T dWbar_k and the dw partial slabs, one pass over the blocked dWbar_k of every piece.
 // slab_add: the launch covers only part of the parameters, so its dw sums are added to the slabs.
 static int launch_stage2(const lory_dims& D, const WsPtrs& q, const AdjPiece pc[3], bool slab_add, cudaStream_t st) {
   const int S = D.B * (D.L / D.T), E = D.E, Ep = e_pad(D);
+  if (adjoint_streams(D)) return launch_adjoint_stream(D, q, pc, slab_add, st);
   int R[3], C[3], first = -1;
   for (int k = 0; k < 3; ++k) {
     R[k] = pc[k].R;
@@ -450,7 +529,6 @@ static int launch_stage2(const lory_dims& D, const WsPtrs& q, const AdjPiece pc[
   p.S = S_launch; p.S_total = S; p.E = E; p.Epad16 = e_pad16(D); p.s_tiles = (S_launch + 127) / 128;
   p.dw_partial = q.dw_partial; p.status = q.status;
   p.slab_add = slab_add ? 1 : 0;
-  p.rpt_shift = stage2_rpt_shift(D);
   p.ncb = stage2_ncb(D);
   stage2_tiles(D, R, C, p.ctiles, p.tile_end);
   for (int k = 0; k < 3; ++k)
@@ -474,7 +552,7 @@ static int launch_stage2(const lory_dims& D, const WsPtrs& q, const AdjPiece pc[
   }
   for (int k = 0; k < 3; ++k) {
     const AdjPiece& a = pc[R[k] > 0 ? k : first];  // an absent piece has no tiles; its maps repeat a present one
-    LORY_TRY(make_blocked_map(&maps.dwbar[k], a.dsrc, a.R, a.C, S, 1, seg_box, p.rpt_shift ? 1 : p.ncb, 1));
+    LORY_TRY(make_blocked_map(&maps.dwbar[k], a.dsrc, a.R, a.C, S, 1, seg_box, p.ncb, 1));
     LORY_TRY(make_expert_map(&maps.theta[k], a.wsrc, a.R, a.C, E, p.Epad16, a.e_stride, a.row_stride));
     LORY_TRY(make_expert_map(&maps.out[k], a.ddst, a.R, a.C, E, E < 32 ? (uint32_t)E : 32u, a.e_stride, a.row_stride));  // no box rows past the experts
     p.acc_base[k] = a.ddst;
@@ -512,12 +590,14 @@ static int launch_stage2(const lory_dims& D, const WsPtrs& q, const AdjPiece pc[
   return LORY_OK;
 }
 
-void tc_split_tables(const lory_dims& D, const Layout& Lo, char* ws, bf16** hi, bf16** lo, bf16** comb, int* Epad) {
+void tc_split_tables(const lory_dims& D, const Layout& Lo, char* ws, bf16** hi, bf16** lo, bf16** comb, int* Epad, bf16** frag) {
   const WsPtrs q = ws_ptrs(D, Lo, ws);
-  *hi = q.w_hi;
-  *lo = q.w_lo;
-  *comb = D.E <= 32 ? q.w_comb : nullptr;
+  const bool rows = !adjoint_streams(D);   // only the tcgen05 adjoint reads the row tables
+  *hi = rows ? q.w_hi : nullptr;
+  *lo = rows ? q.w_lo : nullptr;
+  *comb = rows && D.E <= 32 ? q.w_comb : nullptr;
   *Epad = e_pad(D);
+  *frag = q.w_frag;
 }
 
 int tc_ffn_forward(const lory_dims& D, const Layout& Lo, char* ws, const bf16* x, const bf16* w1, const bf16* w2,
@@ -528,7 +608,7 @@ int tc_ffn_forward(const lory_dims& D, const Layout& Lo, char* ws, const bf16* x
   if (!(D.flags & LORY_FLAG_REUSE_MERGED)) {
     if (!w_is_split) {
       prof_begin("split_w", st);
-      split_w_kernel<<<(unsigned)ceil_div((long)S * (E <= 32 ? 192 : Ep), 256), 256, 0, st>>>(q.w, q.w_hi, q.w_lo, q.w_comb, S, E, Ep);
+      split_w_kernel<<<(unsigned)ceil_div((long)S * (E <= 32 ? 192 : (E + 15) / 16 * 16), 256), 256, 0, st>>>(q.w, q.w_hi, q.w_lo, q.w_comb, q.w_frag, S, E, Ep);
       prof_end(st);
       LORY_AFTER_LAUNCH();
     }

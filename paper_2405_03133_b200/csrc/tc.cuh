@@ -14,12 +14,15 @@ size_t tc_blocked_elems(const lory_dims& D, int R, int C);
 // Elements of the buffer the chunked adjoint (LORY_FLAG_CHUNKED_ADJOINT) keeps one rectangle of per-segment weight
 // gradients in: sized from the device's L2 (environment variable LORY_ADJOINT_CHUNK_MB overrides the budget).
 size_t tc_adjoint_ring_elems(const lory_dims& D);
-// Number of [S,E] partial slabs the tensor-core dw contraction writes.
+// Number of [S,E] partial slabs the tensor-core dw contraction writes, and the most it writes whatever the flags say
+// (gradient accumulation may be asked for on a workspace that was sized without it).
 int tc_dw_slabs(const lory_dims& D);
+int tc_dw_slabs_max(const lory_dims& D);
 
-// Where the bf16 hi / lo tables of the routing weights live in the workspace ([S, *Epad] each), and the
-// combined [S, 64] table (NULL unless E <= 32).  The routing step may fill them directly.
-void tc_split_tables(const lory_dims& D, const Layout& Lo, char* ws, bf16** hi, bf16** lo, bf16** comb, int* Epad);
+// Where the bf16 hi / lo tables of the routing weights live in the workspace ([S, *Epad] each), the combined [S, 192]
+// table (NULL unless E <= 32) - all three NULL where nothing reads them - and the merge's fragments (w_frag_offset).
+// The routing step may fill them directly.
+void tc_split_tables(const lory_dims& D, const Layout& Lo, char* ws, bf16** hi, bf16** lo, bf16** comb, int* Epad, bf16** frag);
 
 // Merge + merged SwiGLU FFN forward (Eq. 2; Section 3.1).  ws holds the regions of Lo.
 // w_is_split: the hi / lo tables are already filled (else they are derived here from the fp32 weights).
