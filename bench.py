@@ -107,7 +107,6 @@ def implementation_bytes(wl):
         "dw": 2 * (S * P1 + E * P1),
         "stage2": 3 * 2 * (S * P1 + (3 * launches_256 - 1) * E * P1),   # read dWbar and W, write (re-read) dW
         "pool_router": 2 * tok * d,
-        "add_pool_grad": 4 * tok * d,
         # grouped GEMMs: operands once + outputs once
         "gemm1_swiglu": 2 * (tok * d + 2 * S * P1 + 3 * tok * f),   # x, Wbar1, Wbar3 -> G, U, H
         "gemm2": 2 * (tok * f + S * P1 + tok * d),                  # H, Wbar2 -> y

@@ -1,7 +1,6 @@
 // The layer inside a pre-norm residual block (the LLaMA block of Section 4.1):  y = x + Lory(RMSNorm(x)).
 // RMSNorm(x) = x / sqrt(mean_j x_j^2 + eps) * gamma per token; all arithmetic in fp32.
-// The forward residual is added in the epilogue of the last GEMM of the layer (tensor-core pipeline) or by
-// residual_add_kernel (plain-FMA pipeline); the backward residual rides in the RMSNorm backward kernel.
+// The forward residual is added in the epilogue of the last GEMM of the layer; the backward residual rides in the RMSNorm backward kernel.
 #include "block.cuh"
 
 namespace lory {
@@ -90,13 +89,6 @@ __global__ void __launch_bounds__(256) rmsnorm_kernel(const T* __restrict__ x, c
       for (int j = lane; j < d; j += 32) out[j] = from_f32<T>(to_f32(row[j]) * inv * to_f32(gamma[j]));
     }
   }
-}
-
-// y += x
-template <typename T>
-__global__ void residual_add_kernel(T* __restrict__ y, const T* __restrict__ x, size_t n) {
-  size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) y[i] = from_f32<T>(to_f32(y[i]) + to_f32(x[i]));
 }
 
 // With n = x * inv, dn = dxh * gamma:  dx = inv * (dn - n * mean_j(dn_j n_j)) + dy  (the residual path),
@@ -237,13 +229,6 @@ int launch_rmsnorm(const T* x, const T* gamma, T* x_hat, float* inv_rms, long to
 }
 
 template <typename T>
-int launch_residual_add(T* y, const T* x, size_t n, cudaStream_t st) {
-  residual_add_kernel<T><<<(unsigned)ceil_div((long)n, 256), 256, 0, st>>>(y, x, n);
-  LORY_AFTER_LAUNCH();
-  return LORY_OK;
-}
-
-template <typename T>
 int launch_rmsnorm_backward(const T* x, const T* gamma, const float* inv_rms, const T* dxh, const T* dy, T* dx,
                             T* dgamma, float* slab, long tokens, int d, int accumulate, cudaStream_t st) {
   const int n_slabs = block_norm_slabs(tokens);
@@ -256,7 +241,6 @@ int launch_rmsnorm_backward(const T* x, const T* gamma, const float* inv_rms, co
 
 #define INST(T)                                                                                                  \
   template int launch_rmsnorm<T>(const T*, const T*, T*, float*, long, int, float, cudaStream_t);                \
-  template int launch_residual_add<T>(T*, const T*, size_t, cudaStream_t);                                       \
   template int launch_rmsnorm_backward<T>(const T*, const T*, const float*, const T*, const T*, T*, T*, float*,  \
                                           long, int, int, cudaStream_t);
 INST(float)

@@ -8,9 +8,6 @@ namespace lory {
 template <typename T>
 int launch_rmsnorm(const T* x, const T* gamma, T* x_hat, float* inv_rms, long tokens, int d, float eps,
                    cudaStream_t st);
-// y += x
-template <typename T>
-int launch_residual_add(T* y, const T* x, size_t n, cudaStream_t st);
 // dx = RMSNorm backward of dxh (gradient wrt x_hat) + dy (the residual path); dgamma = sum over tokens of
 // dxh * x * inv_rms (added to the stored value when accumulate != 0).  slab: float [block_norm_slabs(tokens), d].
 template <typename T>

@@ -104,9 +104,9 @@ static Layout make_layout(const lory_dims& D) {
     Lo.dwbar2 = take(n2 * es);
   }
   Lo.k_chunk = 8192;
-  int simt_slabs = 3 * (int)ceil_div((long)P1, Lo.k_chunk);
-  Lo.n_slabs = use_tc(D) ? tc_dw_slabs(D) : simt_slabs;
-  Lo.dw_partial = take((size_t)(use_tc(D) ? tc_dw_slabs_max(D) : simt_slabs) * S * D.E * 4);
+  const int simt_slabs = fma_merge_supported((int)S, D.E) ? fma_adjoint_slabs((long)P1) : 3 * (int)ceil_div((long)P1, Lo.k_chunk);
+  Lo.n_slabs = blk ? tc_dw_slabs(D) : simt_slabs;
+  Lo.dw_partial = take((size_t)(blk ? tc_dw_slabs_max(D) : simt_slabs) * S * D.E * 4);
   Lo.dw = take(S * D.E * 4);
   Lo.dz = take(S * D.E * 4);
   Lo.dh_bar = take(S * D.d * 4);
@@ -142,18 +142,20 @@ static int check_device() {
 // Plain-FMA pipeline (fp32 mode, and bf16 with LORY_FLAG_SIMT).
 // ---------------------------------------------------------------------------------------
 template <typename T>
-struct Simt {
-  static int g_wTT(const SimtGemm& g, cudaStream_t st) { return launch_simt_gemm<float, T, T>(g, st); }
-  static int g_TTT(const SimtGemm& g, cudaStream_t st) { return launch_simt_gemm<T, T, T>(g, st); }
-  static int g_TTf(const SimtGemm& g, cudaStream_t st) { return launch_simt_gemm<T, T, float>(g, st); }
-};
+static FmaMerge<T> fma_merge_params(const lory_dims& D, const Layout& Lo, char* ws, const T* w1, const T* w2, const T* w3) {
+  FmaMerge<T> m = {};
+  m.w[0] = w1; m.w[1] = w3; m.w[2] = w2;
+  m.route = (const float*)(ws + Lo.w);
+  m.n = (long)D.f * D.d; m.S = D.B * (D.L / D.T); m.E = D.E;
+  return m;
+}
 
 // Field order of SimtGemm: A B C | M N K groups | a_m a_k a_g | b_k b_n b_g | c_m c_n c_g | k_chunk accumulate
 template <typename T>
 static int simt_ffn_forward(const lory_dims& D, const Layout& Lo, char* ws, const T* x, const T* w1, const T* w2,
-                            const T* w3, T* y, cudaStream_t st) {
+                            const T* w3, T* y, cudaStream_t st, const T* residual) {
   const int S = D.B * (D.L / D.T), Tn = D.T, d = D.d, f = D.f, E = D.E;
-  const long P1 = (long)f * d, PS = Lo.seg_stride;
+  const long P1 = (long)f * d, PS = Lo.seg_stride, td = (long)Tn * d, tf = (long)Tn * f;
   const float* w = (const float*)(ws + Lo.w);
   T* wbar1 = (T*)(ws + Lo.wbar1);
   T* wbar3 = (T*)(ws + Lo.wbar3);
@@ -162,37 +164,44 @@ static int simt_ffn_forward(const lory_dims& D, const Layout& Lo, char* ws, cons
   T* U = (T*)(ws + Lo.U);
   T* H = (T*)(ws + Lo.H);
   // merge: Wbar_k[S, P1] = w[S, E] . W_k[E, P1]   (Eq. 2)
-  const T* src[3] = {w1, w3, w2};
-  T* dst[3] = {wbar1, wbar3, wbar2};
-  for (int k = 0; k < 3 && !(D.flags & LORY_FLAG_REUSE_MERGED); ++k) {
-    SimtGemm g = {w, src[k], dst[k], S, (int)P1, E, 1, E, 1, 0, P1, 1, 0, PS, 1, 0, 0, 0};
-    LORY_TRY(Simt<T>::g_wTT(g, st));
+  if (!(D.flags & LORY_FLAG_REUSE_MERGED)) {
+    if (fma_merge_supported(S, E)) {
+      FmaMerge<T> m = fma_merge_params(D, Lo, ws, w1, w2, w3);
+      m.wbar[0] = wbar1; m.wbar[1] = wbar3; m.wbar[2] = wbar2;
+      ProfScope ps("merge", st);
+      LORY_TRY(launch_fma_merge<T>(m, st));
+    } else {
+      const T* src[3] = {w1, w3, w2};
+      T* dst[3] = {wbar1, wbar3, wbar2};
+      for (int k = 0; k < 3; ++k) {
+        SimtGemm g = {w, src[k], dst[k], S, (int)P1, E, 1, E, 1, 0, P1, 1, 0, PS, 1, 0, 0, 0};
+        ProfScope ps("merge", st);
+        LORY_TRY((launch_simt_gemm<float, T, T>(g, st)));
+      }
+    }
   }
-  // G = X Wbar1^T, U = X Wbar3^T, per segment
+  // G = X Wbar1^T, U = X Wbar3^T, H = silu(G) * U, per segment
+  FmaJob j = {};
+  j.A0 = x; j.B0 = wbar1; j.B1 = wbar3; j.C0 = G; j.C1 = U; j.C2 = H;
+  j.M = Tn; j.N = f; j.K = d; j.lda = d; j.ldb = d; j.ldc = f; j.a_g = td; j.b_g = PS; j.c_g = tf;
   {
-    SimtGemm g = {x, wbar1, G, Tn, f, d, S, d, 1, (long)Tn * d, 1, d, PS, f, 1, (long)Tn * f, 0, 0};
-    LORY_TRY(Simt<T>::g_TTT(g, st));
-    g.B = wbar3;
-    g.C = U;
-    LORY_TRY(Simt<T>::g_TTT(g, st));
+    ProfScope ps("gemm1_swiglu", st);
+    LORY_TRY(fma_gemm_swiglu<T>(j, S, st));
   }
-  LORY_TRY(launch_swiglu_fwd<T>(G, U, H, (size_t)S * Tn * f, st));
-  // Y = H Wbar2^T
-  {
-    SimtGemm g = {H, wbar2, y, Tn, d, f, S, f, 1, (long)Tn * f, 1, f, PS, d, 1, (long)Tn * d, 0, 0};
-    LORY_TRY(Simt<T>::g_TTT(g, st));
-  }
-  return LORY_OK;
+  // Y = H Wbar2^T (+ the block's skip connection)
+  j = FmaJob{};
+  j.A0 = H; j.B0 = wbar2; j.C0 = y; j.E0 = residual;
+  j.M = Tn; j.N = d; j.K = f; j.lda = f; j.ldb = f; j.ldc = d; j.a_g = tf; j.b_g = PS; j.c_g = td;
+  ProfScope ps("gemm2", st);
+  return fma_gemm_nt<T>(j, S, st);
 }
 
 template <typename T>
 static int simt_ffn_backward(const lory_dims& D, const Layout& Lo, char* ws, const T* x, const T* w1, const T* w2,
-                             const T* w3, const T* dy, T* dx, T* dw1, T* dw2, T* dw3, cudaStream_t st) {
+                             const T* w3, const T* dy, T* dw1, T* dw2, T* dw3, cudaStream_t st) {
   const int S = D.B * (D.L / D.T), Tn = D.T, d = D.d, f = D.f, E = D.E;
-  const long P1 = (long)f * d, PS = Lo.seg_stride;
+  const long P1 = (long)f * d, PS = Lo.seg_stride, td = (long)Tn * d, tf = (long)Tn * f;
   const float* w = (const float*)(ws + Lo.w);
-  T* wbar1 = (T*)(ws + Lo.wbar1);
-  T* wbar3 = (T*)(ws + Lo.wbar3);
   T* wbar2 = (T*)(ws + Lo.wbar2);
   T* G = (T*)(ws + Lo.G);
   T* U = (T*)(ws + Lo.U);
@@ -203,90 +212,92 @@ static int simt_ffn_backward(const lory_dims& D, const Layout& Lo, char* ws, con
   T* dwbar3 = (T*)(ws + Lo.dwbar3);
   T* dwbar2 = (T*)(ws + Lo.dwbar2);
   float* dw_partial = (float*)(ws + Lo.dw_partial);
-  // dH = dY Wbar2 (into dG), then the SwiGLU backward in place
+  // dH = dY Wbar2, through the SwiGLU: dG, dU
+  FmaJob j = {};
+  j.A0 = dy; j.B0 = wbar2; j.C0 = dG; j.C1 = dU; j.E0 = G; j.E1 = U;
+  j.M = Tn; j.N = f; j.K = d; j.lda = d; j.ldb = f; j.ldc = f; j.a_g = td; j.b_g = PS; j.c_g = tf;
   {
-    SimtGemm g = {dy, wbar2, dG, Tn, f, d, S, d, 1, (long)Tn * d, f, 1, PS, f, 1, (long)Tn * f, 0, 0};
-    LORY_TRY(Simt<T>::g_TTT(g, st));
+    ProfScope ps("dh_dswiglu", st);
+    LORY_TRY(fma_gemm_dswiglu<T>(j, S, st));
   }
-  LORY_TRY(launch_swiglu_bwd<T>(G, U, dG, dU, (size_t)S * Tn * f, st));
-  // dWbar2 = dY^T H  [d, f]
+  // dWbar2 = dY^T H [d, f], dWbar1 = dG^T X, dWbar3 = dU^T X [f, d]
+  FmaJob q[3] = {};
+  const T* a_src[3] = {dG, dU, dy};
+  const T* b_src[3] = {x, x, H};
+  T* o_dst[3] = {dwbar1, dwbar3, dwbar2};
+  for (int k = 0; k < 3; ++k) {
+    const int R = k < 2 ? f : d, C = k < 2 ? d : f;
+    q[k].A0 = a_src[k]; q[k].B0 = b_src[k]; q[k].C0 = o_dst[k];
+    q[k].M = R; q[k].N = C; q[k].K = Tn; q[k].lda = R; q[k].ldb = C; q[k].ldc = C;
+    q[k].a_g = (long)Tn * R; q[k].b_g = (long)Tn * C; q[k].c_g = PS;
+  }
   {
-    SimtGemm g = {dy, H, dwbar2, d, f, Tn, S, 1, d, (long)Tn * d, f, 1, (long)Tn * f, f, 1, PS, 0, 0};
-    LORY_TRY(Simt<T>::g_TTT(g, st));
+    ProfScope ps("wgrad", st);
+    LORY_TRY(fma_gemm_tn<T>(q, S, st));
   }
-  // dWbar1 = dG^T X, dWbar3 = dU^T X  [f, d]
-  {
-    SimtGemm g = {dG, x, dwbar1, f, d, Tn, S, 1, f, (long)Tn * f, d, 1, (long)Tn * d, d, 1, PS, 0, 0};
-    LORY_TRY(Simt<T>::g_TTT(g, st));
-    g.A = dU;
-    g.C = dwbar3;
-    LORY_TRY(Simt<T>::g_TTT(g, st));
-  }
-  // dX = dG Wbar1 + dU Wbar3
-  {
-    SimtGemm g = {dG, wbar1, dx, Tn, d, f, S, f, 1, (long)Tn * f, d, 1, PS, d, 1, (long)Tn * d, 0, 0};
-    LORY_TRY(Simt<T>::g_TTT(g, st));
-    g.A = dU;
-    g.B = wbar3;
-    g.accumulate = 1;
-    LORY_TRY(Simt<T>::g_TTT(g, st));
-  }
-  // adjoint of the merge: dW_k[E, P1] = w^T[E, S] . dWbar_k[S, P1]
-  // and dw[S, E] += dWbar_k[S, P1] . W_k^T[P1, E]  (K split into slabs)
-  const T* dsrc[3] = {dwbar1, dwbar3, dwbar2};
-  const T* wsrc[3] = {w1, w3, w2};
+  // adjoint of the merge: dW_k[E, P1] = w^T[E, S] . dWbar_k[S, P1] and dw[S, E] += dWbar_k[S, P1] . W_k^T[P1, E]
+  const int accumulate = (D.flags & LORY_FLAG_ACCUMULATE_GRADS) ? 1 : 0;
   T* ddst[3] = {dw1, dw3, dw2};
+  if (fma_merge_supported(S, E)) {
+    FmaMerge<T> m = fma_merge_params(D, Lo, ws, w1, w2, w3);
+    for (int k = 0; k < 3; ++k) {
+      m.wbar[k] = o_dst[k];
+      m.dw[k] = ddst[k];
+    }
+    m.slabs = dw_partial;
+    m.accumulate = accumulate;
+    ProfScope ps("stage2", st);
+    return launch_fma_adjoint<T>(m, st);
+  }
+  const T* wsrc[3] = {w1, w3, w2};
   const int slabs_per = (int)ceil_div(P1, Lo.k_chunk);
   for (int k = 0; k < 3; ++k) {
-    SimtGemm g = {w, dsrc[k], ddst[k], E, (int)P1, S, 1, 1, E, 0, PS, 1, 0, P1, 1, 0, 0,
-                  (D.flags & LORY_FLAG_ACCUMULATE_GRADS) ? 1 : 0};
-    LORY_TRY(Simt<T>::g_wTT(g, st));
-    SimtGemm h = {dsrc[k], wsrc[k], dw_partial + (size_t)k * slabs_per * S * E, S, E, (int)P1, slabs_per,
+    SimtGemm g = {w, o_dst[k], ddst[k], E, (int)P1, S, 1, 1, E, 0, PS, 1, 0, P1, 1, 0, 0, accumulate};
+    ProfScope ps("stage2", st);
+    LORY_TRY((launch_simt_gemm<float, T, T>(g, st)));
+    SimtGemm h = {o_dst[k], wsrc[k], dw_partial + (size_t)k * slabs_per * S * E, S, E, (int)P1, slabs_per,
                   PS, 1, 0, 1, P1, 0, E, 1, (long)S * E, Lo.k_chunk, 0};
-    LORY_TRY(Simt<T>::g_TTf(h, st));
+    LORY_TRY((launch_simt_gemm<T, T, float>(h, st)));
   }
   return LORY_OK;
+}
+
+// dX = dG Wbar1 + dU Wbar3 + dh_bar / T (the mean-pool gradient of the router path rides in the epilogue)
+template <typename T>
+static int simt_ffn_backward_dx(const lory_dims& D, const Layout& Lo, char* ws, T* dx, cudaStream_t st) {
+  const int S = D.B * (D.L / D.T), Tn = D.T, d = D.d, f = D.f;
+  FmaJob j = {};
+  j.A0 = ws + Lo.dG; j.A1 = ws + Lo.dU; j.B0 = ws + Lo.wbar1; j.B1 = ws + Lo.wbar3; j.C0 = dx;
+  j.M = Tn; j.N = d; j.K = f; j.lda = f; j.ldb = d; j.ldc = d;
+  j.a_g = (long)Tn * f; j.b_g = Lo.seg_stride; j.c_g = (long)Tn * d;
+  ProfScope ps("dx", st);
+  return fma_gemm_dx<T>(j, S, (const float*)(ws + Lo.dh_bar), 1.0f / (float)Tn, st);
 }
 
 // ---------------------------------------------------------------------------------------
 // Whole-layer drivers
 // ---------------------------------------------------------------------------------------
-// residual (optional): y = residual + layer output.  The tensor-core pipeline adds it in its last GEMM's epilogue,
-// the plain-FMA pipeline with a separate kernel.
+// residual (optional): y = residual + layer output, added in the epilogue of the last GEMM.
 static int run_ffn_forward(const lory_dims& D, const Layout& Lo, char* ws, const float* x, const float* w1,
                            const float* w2, const float* w3, float* y, cudaStream_t st, bool, const float* residual) {
-  {
-    ProfScope ps("simt_forward", st);
-    LORY_TRY(simt_ffn_forward<float>(D, Lo, ws, x, w1, w2, w3, y, st));
-  }
-  if (!residual) return LORY_OK;
-  ProfScope ps("residual_add", st);
-  return launch_residual_add<float>(y, residual, (size_t)D.B * D.L * D.d, st);
+  return simt_ffn_forward<float>(D, Lo, ws, x, w1, w2, w3, y, st, residual);
 }
 static int run_ffn_forward(const lory_dims& D, const Layout& Lo, char* ws, const bf16* x, const bf16* w1,
                            const bf16* w2, const bf16* w3, bf16* y, cudaStream_t st, bool w_is_split,
                            const bf16* residual) {
   if (use_tc(D)) return tc_ffn_forward(D, Lo, ws, x, w1, w2, w3, y, st, w_is_split, residual);
-  {
-    ProfScope ps("simt_forward", st);
-    LORY_TRY(simt_ffn_forward<bf16>(D, Lo, ws, x, w1, w2, w3, y, st));
-  }
-  if (!residual) return LORY_OK;
-  ProfScope ps("residual_add", st);
-  return launch_residual_add<bf16>(y, residual, (size_t)D.B * D.L * D.d, st);
+  return simt_ffn_forward<bf16>(D, Lo, ws, x, w1, w2, w3, y, st, residual);
 }
 static int run_ffn_backward(const lory_dims& D, const Layout& Lo, char* ws, const float* x, const float* w1,
-                            const float* w2, const float* w3, const float* dy, float* dx, float* dw1, float* dw2,
-                            float* dw3, cudaStream_t st) {
-  ProfScope ps("simt_backward", st);
-  return simt_ffn_backward<float>(D, Lo, ws, x, w1, w2, w3, dy, dx, dw1, dw2, dw3, st);
+                            const float* w2, const float* w3, const float* dy, float* dw1, float* dw2, float* dw3,
+                            cudaStream_t st) {
+  return simt_ffn_backward<float>(D, Lo, ws, x, w1, w2, w3, dy, dw1, dw2, dw3, st);
 }
 static int run_ffn_backward(const lory_dims& D, const Layout& Lo, char* ws, const bf16* x, const bf16* w1,
-                            const bf16* w2, const bf16* w3, const bf16* dy, bf16* dx, bf16* dw1, bf16* dw2,
-                            bf16* dw3, cudaStream_t st) {
+                            const bf16* w2, const bf16* w3, const bf16* dy, bf16* dw1, bf16* dw2, bf16* dw3,
+                            cudaStream_t st) {
   if (use_tc(D)) return tc_ffn_backward(D, Lo, ws, x, w1, w2, w3, dy, dw1, dw2, dw3, st);
-  ProfScope ps("simt_backward", st);
-  return simt_ffn_backward<bf16>(D, Lo, ws, x, w1, w2, w3, dy, dx, dw1, dw2, dw3, st);
+  return simt_ffn_backward<bf16>(D, Lo, ws, x, w1, w2, w3, dy, dw1, dw2, dw3, st);
 }
 
 template <typename T>
@@ -322,20 +333,19 @@ static int backward_impl(const lory_dims& D, const Layout& Lo, const T* x, const
                          const T* w3, const T* dy, T* dx, T* dw_r, T* dw1, T* dw2, T* dw3, float* d_route_w,
                          char* ws, cudaStream_t st) {
   const int N = D.L / D.T;
-  LORY_TRY(run_ffn_backward(D, Lo, ws, x, w1, w2, w3, dy, dx, dw1, dw2, dw3, st));
-  ProfScope ps("router_backward", st);
-  LORY_TRY(launch_router_backward<T>((const float*)(ws + Lo.dw_partial), Lo.n_slabs, (const float*)(ws + Lo.p),
-                                     (const float*)(ws + Lo.h_bar), w_r, (float*)(ws + Lo.dw), d_route_w,
-                                     (float*)(ws + Lo.dz), (float*)(ws + Lo.dh_bar), dw_r, D.B, N, D.d, D.E,
-                                     ((D.flags & LORY_FLAG_PREFIX_ROUTING) ? 1 : 0) |
-                                         ((D.flags & LORY_FLAG_FIRST_SEGMENT_GRAD) ? 2 : 0) |
-                                         ((D.flags & LORY_FLAG_ACCUMULATE_GRADS) ? 4 : 0),
-                                     st));
-  prof_end(st);
+  LORY_TRY(run_ffn_backward(D, Lo, ws, x, w1, w2, w3, dy, dw1, dw2, dw3, st));
+  {
+    ProfScope ps("router_backward", st);
+    LORY_TRY(launch_router_backward<T>((const float*)(ws + Lo.dw_partial), Lo.n_slabs, (const float*)(ws + Lo.p),
+                                       (const float*)(ws + Lo.h_bar), w_r, (float*)(ws + Lo.dw), d_route_w,
+                                       (float*)(ws + Lo.dz), (float*)(ws + Lo.dh_bar), dw_r, D.B, N, D.d, D.E,
+                                       ((D.flags & LORY_FLAG_PREFIX_ROUTING) ? 1 : 0) |
+                                           ((D.flags & LORY_FLAG_FIRST_SEGMENT_GRAD) ? 2 : 0) |
+                                           ((D.flags & LORY_FLAG_ACCUMULATE_GRADS) ? 4 : 0),
+                                       st));
+  }
   if (use_tc(D)) return tc_ffn_backward_dx(D, Lo, ws, (const float*)(ws + Lo.dh_bar), (bf16*)dx, st);
-  prof_begin("add_pool_grad", st);
-  LORY_TRY(launch_add_pool_grad<T>(dx, (const float*)(ws + Lo.dh_bar), D.B * D.L, D.T, D.d, st));
-  return LORY_OK;
+  return simt_ffn_backward_dx<T>(D, Lo, ws, dx, st);
 }
 
 }  // namespace lory

@@ -353,18 +353,6 @@ __global__ void __launch_bounds__(512) dwr_kernel(const float* __restrict__ dz, 
   }
 }
 
-// dx[t, j] += dh_bar[s(t), j] / T   (mean-pool backward), fp32 add then round to storage.
-template <typename T>
-__global__ void add_pool_grad_kernel(T* __restrict__ dx, const float* __restrict__ dh_bar, int Tseg, int d,
-                                     size_t total) {
-  size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= total) return;
-  size_t t = i / d;
-  int j = (int)(i - t * d);
-  size_t s = t / Tseg;
-  dx[i] = from_f32<T>(to_f32(dx[i]) + dh_bar[s * d + j] / (float)Tseg);
-}
-
 // ---------------------------------------------------------------------------------------
 // Host launchers
 // ---------------------------------------------------------------------------------------
@@ -394,14 +382,6 @@ int launch_router_backward(const float* dw_partial, int n_slabs, const float* p_
   return LORY_OK;
 }
 
-template <typename T>
-int launch_add_pool_grad(T* dx, const float* dh_bar, int tokens, int Tseg, int d, cudaStream_t st) {
-  size_t total = (size_t)tokens * d;
-  add_pool_grad_kernel<T><<<(unsigned)ceil_div((long)total, 256), 256, 0, st>>>(dx, dh_bar, Tseg, d, total);
-  LORY_AFTER_LAUNCH();
-  return LORY_OK;
-}
-
 // one thread per expert; the S weights of an expert are E floats apart
 __global__ void expert_utilization_kernel(const float* __restrict__ route_w, int S, int E, int* __restrict__ counts) {
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
@@ -422,8 +402,7 @@ int launch_expert_utilization(const float* route_w, int S, int E, int* counts, c
   template int launch_pool_router<T>(const T*, const T*, float*, float*, float*, float*, int, int, int, int, \
                                      int, int, cudaStream_t, RouteExtra);                                    \
   template int launch_router_backward<T>(const float*, int, const float*, const float*, const T*, float*,    \
-                                         float*, float*, float*, T*, int, int, int, int, int, cudaStream_t); \
-  template int launch_add_pool_grad<T>(T*, const float*, int, int, int, cudaStream_t);
+                                         float*, float*, float*, T*, int, int, int, int, int, cudaStream_t);
 INST(float)
 INST(bf16)
 #undef INST

@@ -32,10 +32,6 @@ int launch_router_backward(const float* dw_partial, int n_slabs, const float* p_
                            const T* w_r, float* dw, float* d_route_w, float* dz, float* dh_bar, T* dw_r,
                            int B, int N, int d, int E, int prefix, cudaStream_t st);
 
-// dx[t,:] += dh_bar[segment(t),:] / T
-template <typename T>
-int launch_add_pool_grad(T* dx, const float* dh_bar, int tokens, int Tseg, int d, cudaStream_t st);
-
 // counts[e] = number of segments whose routing weight for expert e exceeds 2/E
 // (the activation criterion of the paper's expert-utilisation analysis).
 int launch_expert_utilization(const float* route_w, int S, int E, int* counts, cudaStream_t st);

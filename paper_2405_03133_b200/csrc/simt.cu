@@ -1,5 +1,7 @@
 #include "simt.cuh"
 
+#include <type_traits>
+
 namespace lory {
 
 template <typename TA, typename TB, typename TC>
@@ -84,45 +86,296 @@ int launch_simt_gemm(const SimtGemm& g, cudaStream_t st) {
   return LORY_OK;
 }
 
-template <typename T>
-__global__ void swiglu_fwd_kernel(const T* __restrict__ G, const T* __restrict__ U, T* __restrict__ H, size_t n) {
-  size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  float g = to_f32(G[i]), u = to_f32(U[i]);
-  H[i] = from_f32<T>(g * sigmoidf_(g) * u);
+// ---------------------------------------------------------------------------------------
+// FFN contractions
+// ---------------------------------------------------------------------------------------
+static int sm_count_simt() {
+  static int n[64];
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) dev = 0;
+  if (!n[dev] && (cudaDeviceGetAttribute(&n[dev], cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n[dev] <= 0)) n[dev] = 148;
+  return n[dev];
 }
 
+// Tile choice.  128-row tiles have the best ratio of FMAs to shared-memory reads and need enough of them; below two per
+// SM 64-row tiles, below one per SM 32-row tiles (d = 256, f = 688, 8 segments of 128: dx 109, 60 and 44 us).  Two k-groups
+// per CTA where an SM gets fewer than three CTAs, and always with 32 rows, where a thread has too few FMAs between its
+// shared-memory reads to hide them (16-token segments, d = 301: 168 -> 136 us).
+template <typename T, bool A_K, bool B_K, int MODE, int EPI>
+static int fma_launch(FmaArgs a, int groups, cudaStream_t st) {
+  constexpr int TILE_N = MODE == FMA_DUALB ? 32 : 64;
+  const int sms = sm_count_simt();
+  auto count = [&](int bm) {
+    long t = 0;
+    for (int i = 0; i < a.jobs; ++i) t += ceil_div(a.job[i].M, bm) * ceil_div(a.job[i].N, TILE_N) * groups;
+    return t;
+  };
+  int mmax = 0;
+  for (int i = 0; i < a.jobs; ++i) mmax = a.job[i].M > mmax ? a.job[i].M : mmax;
+  const int bm = (mmax > 64 && count(128) >= 2L * sms) ? 128 : ((mmax > 32 && count(64) >= sms) ? 64 : 32);
+  const long tiles = count(bm);
+  if (tiles <= 0) return LORY_OK;
+  if (tiles > 0x7fffffffL) return LORY_ERR_SHAPE;
+  int acc = 0;
+  bool vec = true;
+  for (int i = 0; i < a.jobs; ++i) {
+    FmaJob& j = a.job[i];
+    j.m_tiles = (int)ceil_div(j.M, bm);
+    j.n_tiles = (int)ceil_div(j.N, TILE_N);
+    acc += j.m_tiles * j.n_tiles * groups;
+    j.tile_end = acc;
+    const uintptr_t out = (uintptr_t)j.C0 | (uintptr_t)j.C1 | (uintptr_t)j.C2 | (uintptr_t)j.E0 | (uintptr_t)j.E1;
+    j.vec = j.ldc % 4 == 0 && j.c_g % 4 == 0 && out % (4 * sizeof(T)) == 0;
+    const uintptr_t in = (uintptr_t)j.A0 | (uintptr_t)j.A1 | (uintptr_t)j.B0 | (uintptr_t)j.B1;
+    vec = vec && j.lda % 4 == 0 && j.ldb % 4 == 0 && j.a_g % 4 == 0 && j.b_g % 4 == 0 && in % (4 * sizeof(T)) == 0 &&
+          (A_K ? j.K : j.M) % 4 == 0 && (B_K ? j.K : j.N) % 4 == 0;
+  }
+  auto pick = [&](auto v) {
+    constexpr bool V = decltype(v)::value;
+    const bool two = bm == 32 || tiles < 3L * sms;
+    if (bm == 128) fma_gemm_kernel<T, A_K, B_K, MODE, EPI, 128, 1, V><<<(unsigned)tiles, 128, 0, st>>>(a);
+    else if (bm == 64 && two) fma_gemm_kernel<T, A_K, B_K, MODE, EPI, 64, 2, V><<<(unsigned)tiles, 256, 0, st>>>(a);
+    else if (bm == 64) fma_gemm_kernel<T, A_K, B_K, MODE, EPI, 64, 1, V><<<(unsigned)tiles, 128, 0, st>>>(a);
+    else fma_gemm_kernel<T, A_K, B_K, MODE, EPI, 32, 2, V><<<(unsigned)tiles, 256, 0, st>>>(a);
+  };
+  if (vec) pick(std::true_type());
+  else pick(std::false_type());
+  LORY_AFTER_LAUNCH();
+  return LORY_OK;
+}
+static FmaArgs one_job(const FmaJob& j) {
+  FmaArgs a = {};
+  a.job[0] = j;
+  a.jobs = 1;
+  return a;
+}
 template <typename T>
-__global__ void swiglu_bwd_kernel(const T* __restrict__ G, const T* __restrict__ U, T* __restrict__ dG,
-                                  T* __restrict__ dU, size_t n) {
-  size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  float g = to_f32(G[i]), u = to_f32(U[i]), dh = to_f32(dG[i]);
-  float sig = sigmoidf_(g);
-  dG[i] = from_f32<T>(dh * u * sig * (1.0f + g * (1.0f - sig)));
-  dU[i] = from_f32<T>(dh * g * sig);
+int fma_gemm_swiglu(FmaJob j, int groups, cudaStream_t st) { return fma_launch<T, true, true, FMA_DUALB, FMA_SWIGLU>(one_job(j), groups, st); }
+template <typename T>
+int fma_gemm_nt(FmaJob j, int groups, cudaStream_t st) { return fma_launch<T, true, true, FMA_PLAIN, FMA_STORE>(one_job(j), groups, st); }
+template <typename T>
+int fma_gemm_dswiglu(FmaJob j, int groups, cudaStream_t st) { return fma_launch<T, true, false, FMA_PLAIN, FMA_DSWIGLU>(one_job(j), groups, st); }
+template <typename T>
+int fma_gemm_tn(const FmaJob (&j)[3], int groups, cudaStream_t st) {
+  FmaArgs a = {};
+  for (int i = 0; i < 3; ++i) a.job[i] = j[i];
+  a.jobs = 3;
+  return fma_launch<T, false, false, FMA_PLAIN, FMA_STORE>(a, groups, st);
+}
+template <typename T>
+int fma_gemm_dx(FmaJob j, int groups, const float* rowvec, float scale, cudaStream_t st) {
+  FmaArgs a = one_job(j);
+  a.rowvec = rowvec;
+  a.row_scale = scale;
+  return fma_launch<T, true, false, FMA_DUALK, FMA_ROWADD>(a, groups, st);
 }
 
+// ---------------------------------------------------------------------------------------
+// Merge: Wbar_k[s, p] = sum_e w[s, e] W_k[e, p].  HBM-bound: 4 (E + S) bytes per parameter.  A thread owns four consecutive
+// parameters and walks the segments 16 at a time; the experts' values come from L1 after the first walk.  grid.y = matrix.
+// ---------------------------------------------------------------------------------------
 template <typename T>
-int launch_swiglu_fwd(const T* G, const T* U, T* H, size_t n, cudaStream_t st) {
-  swiglu_fwd_kernel<T><<<(unsigned)ceil_div((long)n, 256), 256, 0, st>>>(G, U, H, n);
+__global__ void __launch_bounds__(128) fma_merge_kernel(const __grid_constant__ FmaMerge<T> p) {
+  constexpr int SC = 16;
+  __shared__ __align__(16) float s_w[32][SC];  // [expert][segment of the chunk]
+  const int k = blockIdx.y;
+  const long i0 = ((long)blockIdx.x * 128 + threadIdx.x) * 4;
+  const int left = i0 < p.n ? (int)min(4L, p.n - i0) : 0;
+  const bool vec = (p.n & 3) == 0 && (((uintptr_t)p.w[k] | (uintptr_t)p.wbar[k]) & (4 * sizeof(T) - 1)) == 0;
+  for (int s0 = 0; s0 < p.S; s0 += SC) {
+    if (s0 > 0) __syncthreads();
+    for (int i = threadIdx.x; i < p.E * SC; i += 128) {
+      const int e = i / SC, s = s0 + i % SC;
+      s_w[e][i % SC] = s < p.S ? p.route[(size_t)s * p.E + e] : 0.f;
+    }
+    __syncthreads();
+    float acc[SC][4];
+#pragma unroll
+    for (int s = 0; s < SC; ++s) acc[s][0] = acc[s][1] = acc[s][2] = acc[s][3] = 0.f;
+    for (int e = 0; e < p.E; ++e) {
+      float v[4];
+      load4(p.w[k] + (size_t)e * p.n + i0, left, vec, v);
+#pragma unroll
+      for (int s4 = 0; s4 < SC; s4 += 4) {
+        const float4 w = *reinterpret_cast<const float4*>(&s_w[e][s4]);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          acc[s4][i] = fmaf(w.x, v[i], acc[s4][i]);
+          acc[s4 + 1][i] = fmaf(w.y, v[i], acc[s4 + 1][i]);
+          acc[s4 + 2][i] = fmaf(w.z, v[i], acc[s4 + 2][i]);
+          acc[s4 + 3][i] = fmaf(w.w, v[i], acc[s4 + 3][i]);
+        }
+      }
+    }
+#pragma unroll
+    for (int s = 0; s < SC; ++s)
+      if (s0 + s < p.S) store4(p.wbar[k] + (size_t)(s0 + s) * p.n + i0, left, vec, acc[s]);
+  }
+}
+
+// ---------------------------------------------------------------------------------------
+// Adjoint of the merge, one pass over dWbar: dW_k[e, p] = sum_s w[s, e] dWbar_k[s, p] and dw[s, e] += sum_p dWbar_k[s, p]
+// W_k[e, p].  HBM-bound: 4 (S + 2 E) bytes per parameter.  A CTA takes tiles of 256 parameters in turn, 32 segments at a
+// time: a thread owns one parameter for the first product (its dWbar value is in a register); the second runs on the tiles
+// in shared memory, 4 segments x EMAX / 8 experts per thread with the parameters split over four neighbouring lanes.  Rows
+// of 260 floats keep the 16-byte reads of four-apart rows on different banks.  The CTA's dw sums stay in shared memory.
+// ---------------------------------------------------------------------------------------
+static const int kFmaTile = 256, kFmaRow = 260, kFmaSegs = 32;
+static size_t fma_adjoint_smem(int S, int E, int emax) {
+  return ((size_t)(kFmaSegs + emax) * kFmaRow + (size_t)kFmaSegs * emax + (size_t)S * E) * sizeof(float);
+}
+
+template <typename T, int EMAX>
+__global__ void __launch_bounds__(256) fma_adjoint_kernel(const __grid_constant__ FmaMerge<T> p) {
+  constexpr int EB = EMAX / 8;
+  extern __shared__ __align__(16) float s_dyn[];
+  float* s_d = s_dyn;                          // [32 segments][260]
+  float* s_e = s_d + kFmaSegs * kFmaRow;       // [EMAX][260]
+  float* s_w = s_e + EMAX * kFmaRow;           // [32][EMAX] routing weights of the chunk
+  float* s_dw = s_w + kFmaSegs * EMAX;         // [S][E]
+  const int tid = threadIdx.x, ks = tid & 3, sg = (tid >> 2) & 7, eg = tid >> 5;
+  for (int i = tid; i < p.S * p.E; i += 256) s_dw[i] = 0.f;
+  const int per = (int)((p.n + kFmaTile - 1) / kFmaTile), chunks = (p.S + kFmaSegs - 1) / kFmaSegs;
+  // One step = one chunk of segments of one tile.  The next step's values are on their way in registers (ve, vd) while
+  // this one is worked on: 198 -> 128 us at S = 18, E = 6, n = 670 000.
+  float ve[EMAX], vd[kFmaSegs];
+  auto fetch = [&](int tile, int chunk) {
+    const int k = tile / per;
+    const long i0 = (long)(tile - k * per) * kFmaTile + tid;
+    const bool in = i0 < p.n;
+    if (chunk == 0) {
+#pragma unroll
+      for (int e = 0; e < EMAX; ++e) ve[e] = (in && e < p.E) ? to_f32(p.w[k][(size_t)e * p.n + i0]) : 0.f;
+    }
+    const T* d = p.wbar[k] + (size_t)chunk * kFmaSegs * p.n + i0;
+    const int ns = in ? p.S - chunk * kFmaSegs : 0;
+#pragma unroll
+    for (int s = 0; s < kFmaSegs; ++s) vd[s] = s < ns ? to_f32(d[(size_t)s * p.n]) : 0.f;
+  };
+  float acc[EMAX];
+  int tile = blockIdx.x, chunk = 0;
+  if (tile < 3 * per) fetch(tile, 0);
+  while (tile < 3 * per) {
+    const int s0 = chunk * kFmaSegs, ns = min(kFmaSegs, p.S - s0), k = tile / per;
+    const long i0 = (long)(tile - k * per) * kFmaTile + tid;
+    const bool last = chunk + 1 == chunks;
+    __syncthreads();   // the tiles in shared memory have been read
+    if (chunk == 0) {
+#pragma unroll
+      for (int e = 0; e < EMAX; ++e) {
+        s_e[e * kFmaRow + tid] = ve[e];
+        acc[e] = 0.f;
+      }
+    }
+#pragma unroll
+    for (int s = 0; s < kFmaSegs; ++s) s_d[s * kFmaRow + tid] = vd[s];
+    for (int i = tid; i < kFmaSegs * EMAX; i += 256) {
+      const int s = i / EMAX, e = i % EMAX;
+      s_w[i] = (s < ns && e < p.E) ? p.route[(size_t)(s0 + s) * p.E + e] : 0.f;
+    }
+    __syncthreads();
+    const int next_chunk = last ? 0 : chunk + 1, next_tile = last ? tile + (int)gridDim.x : tile;
+    if (next_tile < 3 * per) fetch(next_tile, next_chunk);
+    for (int s = 0; s < ns; ++s) {
+      const float d = s_d[s * kFmaRow + tid];
+#pragma unroll
+      for (int e = 0; e < EMAX; e += 4) {
+        const float4 w = *reinterpret_cast<const float4*>(&s_w[s * EMAX + e]);
+        acc[e] = fmaf(w.x, d, acc[e]);
+        acc[e + 1] = fmaf(w.y, d, acc[e + 1]);
+        acc[e + 2] = fmaf(w.z, d, acc[e + 2]);
+        acc[e + 3] = fmaf(w.w, d, acc[e + 3]);
+      }
+    }
+    if (last && i0 < p.n) {
+#pragma unroll
+      for (int e = 0; e < EMAX; ++e)
+        if (e < p.E) {
+          T* q = p.dw[k] + (size_t)e * p.n + i0;
+          *q = from_f32<T>(p.accumulate ? acc[e] + to_f32(*q) : acc[e]);
+        }
+    }
+    if (sg * 4 < ns && eg * EB < p.E) {
+      float dot[4][EB];
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int e = 0; e < EB; ++e) dot[i][e] = 0.f;
+#pragma unroll 2
+      for (int j = 0; j < kFmaTile / 16; ++j) {
+        float4 d4[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) d4[i] = *reinterpret_cast<const float4*>(&s_d[(sg * 4 + i) * kFmaRow + (j * 4 + ks) * 4]);
+#pragma unroll
+        for (int e = 0; e < EB; ++e) {
+          const float4 w4 = *reinterpret_cast<const float4*>(&s_e[(eg * EB + e) * kFmaRow + (j * 4 + ks) * 4]);
+#pragma unroll
+          for (int i = 0; i < 4; ++i)
+            dot[i][e] = fmaf(d4[i].x, w4.x, fmaf(d4[i].y, w4.y, fmaf(d4[i].z, w4.z, fmaf(d4[i].w, w4.w, dot[i][e]))));
+        }
+      }
+      // the four lanes of a segment group are in here together
+      const unsigned mask = __activemask();
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int e = 0; e < EB; ++e) {
+          float x = dot[i][e];
+          x += __shfl_xor_sync(mask, x, 1);
+          x += __shfl_xor_sync(mask, x, 2);
+          const int s = s0 + sg * 4 + i, ee = eg * EB + e;
+          if (ks == 0 && s < p.S && ee < p.E) s_dw[s * p.E + ee] += x;
+        }
+    }
+    tile = next_tile;
+    chunk = next_chunk;
+  }
+  __syncthreads();
+  float* slab = p.slabs + (size_t)blockIdx.x * p.S * p.E;
+  for (int i = tid; i < p.S * p.E; i += 256) slab[i] = s_dw[i];
+}
+
+bool fma_merge_supported(int S, int E) {
+  return E <= 32 && fma_adjoint_smem(S, E, E <= 8 ? 8 : (E <= 16 ? 16 : 32)) <= 160 * 1024;
+}
+int fma_adjoint_slabs(long n) {
+  const long tiles = 3 * ceil_div(n, kFmaTile), cap = 2L * sm_count_simt();
+  return (int)(tiles < cap ? tiles : cap);
+}
+template <typename T>
+int launch_fma_merge(const FmaMerge<T>& p, cudaStream_t st) {
+  fma_merge_kernel<T><<<dim3((unsigned)ceil_div(p.n, 512), 3), 128, 0, st>>>(p);
+  LORY_AFTER_LAUNCH();
+  return LORY_OK;
+}
+template <typename T, int EMAX>
+static int launch_fma_adjoint_t(const FmaMerge<T>& p, cudaStream_t st) {
+  const size_t smem = fma_adjoint_smem(p.S, p.E, EMAX);
+  LORY_CUDA_OK(cudaFuncSetAttribute(fma_adjoint_kernel<T, EMAX>, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024));
+  fma_adjoint_kernel<T, EMAX><<<fma_adjoint_slabs(p.n), 256, smem, st>>>(p);
   LORY_AFTER_LAUNCH();
   return LORY_OK;
 }
 template <typename T>
-int launch_swiglu_bwd(const T* G, const T* U, T* dG, T* dU, size_t n, cudaStream_t st) {
-  swiglu_bwd_kernel<T><<<(unsigned)ceil_div((long)n, 256), 256, 0, st>>>(G, U, dG, dU, n);
-  LORY_AFTER_LAUNCH();
-  return LORY_OK;
+int launch_fma_adjoint(const FmaMerge<T>& p, cudaStream_t st) {
+  if (p.E <= 8) return launch_fma_adjoint_t<T, 8>(p, st);
+  if (p.E <= 16) return launch_fma_adjoint_t<T, 16>(p, st);
+  return launch_fma_adjoint_t<T, 32>(p, st);
 }
 
 template int launch_simt_gemm<float, float, float>(const SimtGemm&, cudaStream_t);
 template int launch_simt_gemm<float, bf16, bf16>(const SimtGemm&, cudaStream_t);
-template int launch_simt_gemm<bf16, bf16, bf16>(const SimtGemm&, cudaStream_t);
 template int launch_simt_gemm<bf16, bf16, float>(const SimtGemm&, cudaStream_t);
-template int launch_swiglu_fwd<float>(const float*, const float*, float*, size_t, cudaStream_t);
-template int launch_swiglu_fwd<bf16>(const bf16*, const bf16*, bf16*, size_t, cudaStream_t);
-template int launch_swiglu_bwd<float>(const float*, const float*, float*, float*, size_t, cudaStream_t);
-template int launch_swiglu_bwd<bf16>(const bf16*, const bf16*, bf16*, bf16*, size_t, cudaStream_t);
+#define INST(T)                                                                              \
+  template int fma_gemm_swiglu<T>(FmaJob, int, cudaStream_t);                                \
+  template int fma_gemm_nt<T>(FmaJob, int, cudaStream_t);                                    \
+  template int fma_gemm_dswiglu<T>(FmaJob, int, cudaStream_t);                               \
+  template int fma_gemm_tn<T>(const FmaJob (&)[3], int, cudaStream_t);                       \
+  template int fma_gemm_dx<T>(FmaJob, int, const float*, float, cudaStream_t);               \
+  template int launch_fma_merge<T>(const FmaMerge<T>&, cudaStream_t);                        \
+  template int launch_fma_adjoint<T>(const FmaMerge<T>&, cudaStream_t);
+INST(float)
+INST(bf16)
+#undef INST
 
 }  // namespace lory
