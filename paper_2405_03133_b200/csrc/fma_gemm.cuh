@@ -258,7 +258,7 @@ __global__ void __launch_bounds__(128 * KG, 3) fma_gemm_kernel(const __grid_cons
     if (m >= J.M) continue;
     const size_t row = (size_t)g * J.c_g + (size_t)m * J.ldc;
     float v[2][4] = {{acc[r][0].x, acc[r][0].y, acc[r][1].x, acc[r][1].y}, {acc[r][2].x, acc[r][2].y, acc[r][3].x, acc[r][3].y}};
-    if (EPI == FMA_SWIGLU) {
+    if constexpr (EPI == FMA_SWIGLU) {
       const int n = n0 + tx * 4, left = J.N - n;
       if (left <= 0) continue;
       float h[4];
@@ -267,34 +267,34 @@ __global__ void __launch_bounds__(128 * KG, 3) fma_gemm_kernel(const __grid_cons
       store4(static_cast<T*>(J.C0) + row + n, left, vec, v[0]);
       store4(static_cast<T*>(J.C1) + row + n, left, vec, v[1]);
       store4(static_cast<T*>(J.C2) + row + n, left, vec, h);
-      continue;
-    }
+    } else {
 #pragma unroll
-    for (int half = 0; half < 2; ++half) {
-      const int n = n0 + half * 32 + tx * 4, left = J.N - n;
-      if (left <= 0) continue;
-      if (EPI == FMA_DSWIGLU) {
-        float gg[4], uu[4], du[4];
-        load4(static_cast<const T*>(J.E0) + row + n, left, vec, gg);
-        load4(static_cast<const T*>(J.E1) + row + n, left, vec, uu);
+      for (int half = 0; half < 2; ++half) {
+        const int n = n0 + half * 32 + tx * 4, left = J.N - n;
+        if (left <= 0) continue;
+        if (EPI == FMA_DSWIGLU) {
+          float gg[4], uu[4], du[4];
+          load4(static_cast<const T*>(J.E0) + row + n, left, vec, gg);
+          load4(static_cast<const T*>(J.E1) + row + n, left, vec, uu);
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const float s = sigmoidf_(gg[i]), dh = v[half][i];
-          v[half][i] = dh * uu[i] * s * (1.0f + gg[i] * (1.0f - s));
-          du[i] = dh * gg[i] * s;
+          for (int i = 0; i < 4; ++i) {
+            const float s = sigmoidf_(gg[i]), dh = v[half][i];
+            v[half][i] = dh * uu[i] * s * (1.0f + gg[i] * (1.0f - s));
+            du[i] = dh * gg[i] * s;
+          }
+          store4(static_cast<T*>(J.C1) + row + n, left, vec, du);
+        } else if (EPI == FMA_ROWADD) {
+#pragma unroll
+          for (int i = 0; i < 4; ++i)
+            if (i < left) v[half][i] += p.rowvec[(size_t)g * J.N + n + i] * p.row_scale;
+        } else if (J.E0) {
+          float o[4];
+          load4(static_cast<const T*>(J.E0) + row + n, left, vec, o);
+#pragma unroll
+          for (int i = 0; i < 4; ++i) v[half][i] += o[i];
         }
-        store4(static_cast<T*>(J.C1) + row + n, left, vec, du);
-      } else if (EPI == FMA_ROWADD) {
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-          if (i < left) v[half][i] += p.rowvec[(size_t)g * J.N + n + i] * p.row_scale;
-      } else if (J.E0) {
-        float o[4];
-        load4(static_cast<const T*>(J.E0) + row + n, left, vec, o);
-#pragma unroll
-        for (int i = 0; i < 4; ++i) v[half][i] += o[i];
+        store4(static_cast<T*>(J.C0) + row + n, left, vec, v[half]);
       }
-      store4(static_cast<T*>(J.C0) + row + n, left, vec, v[half]);
     }
   }
 }

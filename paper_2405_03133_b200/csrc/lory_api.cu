@@ -305,7 +305,7 @@ static int forward_impl(const lory_dims& D, const Layout& Lo, const T* x, const 
                         const T* w3, T* y, float* route_w, float* route_p, const float* injected_w, char* ws,
                         cudaStream_t st, const T* residual = nullptr) {
   const int N = D.L / D.T, S = D.B * N;
-  LORY_CUDA_OK(cudaMemsetAsync(ws + Lo.status, 0, 256, st));
+  if (!(use_tc(D) && tc_clears_status(D))) LORY_CUDA_OK(cudaMemsetAsync(ws + Lo.status, 0, 256, st));
   float* w = (float*)(ws + Lo.w);
   bool w_is_split = false;
   if (D.flags & LORY_FLAG_REUSE_MERGED) {

@@ -16,6 +16,7 @@
 #include <stdio.h>
 #include <stdlib.h>
 
+#include "decode_tc.cuh"
 #include "gemm_tc.cuh"
 #include "stage2_tc.cuh"
 #include "stream_tc.cuh"
@@ -600,6 +601,70 @@ void tc_split_tables(const lory_dims& D, const Layout& Lo, char* ws, bf16** hi, 
   *frag = q.w_frag;
 }
 
+// Launch attribute of programmatic dependent launch: the kernel may start while its predecessor runs (it waits itself).
+template <typename K, typename P>
+static int launch_pdl(K kern, dim3 grid, int threads, int smem, const P& p, cudaStream_t st) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  LORY_CUDA_OK(cudaLaunchKernelEx(&cfg, kern, p));
+  LORY_AFTER_LAUNCH();
+  return LORY_OK;
+}
+template <int MODE, int NT, int MT>
+static int launch_decode_t(const DecodeParams& p, cudaStream_t st) {
+  using D = Decode<MODE, NT, MT>;
+  static bool attr_set[kMaxDevices];
+  LORY_TRY(allow_dynamic_smem(decode_kernel<MODE, NT, MT>, D::SMEM, attr_set));
+  const long tiles = ceil_div(p.R, D::TR) * p.S, cap = (long)D::CTAS * sm_count();
+  return launch_pdl(decode_kernel<MODE, NT, MT>, dim3((unsigned)(tiles < cap ? tiles : cap)), 256, D::SMEM, p, st);
+}
+// Two weight tiles at a time from 17 tokens on, and below where every CTA still gets three such double tiles (32 sequences,
+// 8 tokens, d = 1024: 109 -> 89 us; with two sequences at d = 2048 the coarser split costs more than it saves: 27 -> 30).
+template <int MODE>
+static int launch_decode_m(const DecodeParams& p, cudaStream_t st) {
+  const bool two = ceil_div(p.R, MODE == DECODE_16 ? 32 : 16) * p.S >= 6L * sm_count();
+  if (p.n <= 8) return two ? launch_decode_t<MODE, 1, 2>(p, st) : launch_decode_t<MODE, 1, 1>(p, st);
+  if (p.n <= 16) return two ? launch_decode_t<MODE, 2, 2>(p, st) : launch_decode_t<MODE, 2, 1>(p, st);
+  if (p.n <= 32) return launch_decode_t<MODE, 4, 2>(p, st);
+  return launch_decode_t<MODE, 8, 2>(p, st);
+}
+// Where the decode kernels run.  Past 16 tokens they fetch as many token as weight bytes, and the grouped GEMMs are the
+// faster ones once these have the tiles to fill the GPU, twice over for up to 32 tokens (d = 1024, f = 2752, 24 tokens, 8
+// sequences: 47 -> 42 us, 16: 72 -> 80; 40 tokens, 4 sequences: 36 -> 30, 8: 47 -> 58).
+static bool decode_supported(const lory_dims& D) {
+  if (!(D.flags & LORY_FLAG_REUSE_MERGED) || D.T > 64) return false;
+  const long gemm_tiles = ceil_div(D.f, 128) * D.B * (D.L / D.T);
+  return D.T <= 16 || gemm_tiles <= (D.T <= 32 ? 2L : 1L) * sm_count();
+}
+bool tc_clears_status(const lory_dims& D) { return decode_supported(D); }
+static int launch_decode(const lory_dims& D, const WsPtrs& q, const bf16* x, bf16* y, cudaStream_t st) {
+  if ((uintptr_t)x & 15) {
+    snprintf(call_state().cuda_error, sizeof(call_state().cuda_error), "x does not start on a 16-byte boundary");
+    return LORY_ERR_CUDA;
+  }
+  DecodeParams p = {};
+  p.wa = q.wbar1; p.wb = q.wbar3; p.x = x; p.out = q.H;
+  p.S = D.B * (D.L / D.T); p.n = D.T; p.R = D.f; p.K = D.d; p.Cb = (D.d + 63) / 64; p.status = q.status;
+  {
+    ProfScope ps("gemm1_swiglu", st);
+    LORY_TRY(launch_decode_m<DECODE_GATE>(p, st));
+  }
+  p.wa = q.wbar2; p.wb = nullptr; p.x = q.H; p.out = y;
+  p.R = D.d; p.K = D.f; p.Cb = (D.f + 63) / 64;
+  ProfScope ps("gemm2", st);
+  // 16-row tiles, or 8-row ones (half of the instruction's rows empty) where those would leave SMs without a CTA
+  if (p.n <= 8 && ceil_div(p.R, 16) * p.S < sm_count()) return launch_decode_t<DECODE_8, 1, 1>(p, st);
+  return launch_decode_m<DECODE_16>(p, st);
+}
+
 int tc_ffn_forward(const lory_dims& D, const Layout& Lo, char* ws, const bf16* x, const bf16* w1, const bf16* w2,
                    const bf16* w3, bf16* y, cudaStream_t st, bool w_is_split, const bf16* residual) {
   const int S = D.B * (D.L / D.T), T = D.T, d = D.d, f = D.f, E = D.E, Ep = e_pad(D);
@@ -617,6 +682,8 @@ int tc_ffn_forward(const lory_dims& D, const Layout& Lo, char* ws, const bf16* x
     bf16* dst[3] = {q.wbar1, q.wbar3, q.wbar2};
     LORY_TRY(launch_merge(D, q, src, dst, st));
   }
+
+  if (decode_supported(D) && !residual) return launch_decode(D, q, x, y, st);
 
   // G = X Wbar1^T, U = X Wbar3^T, H = silu(G) * U, one group per segment
   {

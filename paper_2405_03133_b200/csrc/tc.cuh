@@ -9,6 +9,8 @@ namespace lory {
 size_t tc_w_split_bytes(const lory_dims& D);
 // Whether the tensor-core pipeline covers this problem (else the plain-FMA pipeline runs).
 bool tc_supported(const lory_dims& D);
+// Whether tc_ffn_forward's own kernels clear the status word (else the caller does before it).
+bool tc_clears_status(const lory_dims& D);
 // Elements of the blocked layout of a per-segment [R, C] matrix over all segments.
 size_t tc_blocked_elems(const lory_dims& D, int R, int C);
 // Elements of the buffer the chunked adjoint (LORY_FLAG_CHUNKED_ADJOINT) keeps one rectangle of per-segment weight
