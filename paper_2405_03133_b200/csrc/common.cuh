@@ -56,6 +56,49 @@ struct ProfScope {
   ~ProfScope() { prof_end(st); }
 };
 
+// ---- launches that overlap their predecessor's end (programmatic dependent launch) ----------
+// A kernel launched that way may have its CTAs on the GPU before the kernel in front of it has ended, so
+// that its own set-up (barriers, TMEM, descriptors) and the launch itself cost nothing.  EVERY CTA of such a kernel calls
+// pdl_wait() before it touches global memory: the call returns once the kernel in front has ended and its writes are
+// visible (and so, as that one waited too, everything before it).  pdl_launch() lets the next kernel's CTAs in; it takes
+// effect when all CTAs of the grid have called it or ended, so they never take the place of a CTA that still has to start.
+// Not for a kernel whose split of an SM's memory into L1 and shared memory differs from its predecessor's in a way that
+// matters to it: an SM changes the split only when it is empty, so an overlapped kernel runs with the one it finds
+// (measured: the merge after the routing kernels lost 20 % with the GEMMs' 228 KB of shared memory still set up, the
+// plain-FMA GEMMs 10 % with too little for their CTAs).  Such kernels pass overlap = false, and their pdl_wait() returns
+// at once.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+template <typename... P, typename... A>
+int launch_kernel(bool overlap, void (*kern)(P...), dim3 grid, int threads, size_t smem, cudaStream_t st, int cluster,
+                  A&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3((unsigned)threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[2];
+  cfg.attrs = attr;
+  if (overlap) {
+    attr[cfg.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[cfg.numAttrs++].val.programmaticStreamSerializationAllowed = 1;
+  }
+  if (cluster > 1) {
+    attr[cfg.numAttrs].id = cudaLaunchAttributeClusterDimension;
+    attr[cfg.numAttrs].val.clusterDim.x = (unsigned)cluster;
+    attr[cfg.numAttrs].val.clusterDim.y = 1;
+    attr[cfg.numAttrs++].val.clusterDim.z = 1;
+  }
+  LORY_CUDA_OK(cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...));
+  LORY_AFTER_LAUNCH();
+  return LORY_OK;
+}
+template <typename... P, typename... A>
+int launch_overlapped(void (*kern)(P...), dim3 grid, int threads, size_t smem, cudaStream_t st, int cluster, A&&... args) {
+  return launch_kernel(true, kern, grid, threads, smem, st, cluster, args...);
+}
+
 // ---- storage conversion ---------------------------------------------------------------
 __device__ __forceinline__ float to_f32(float v) { return v; }
 __device__ __forceinline__ float to_f32(bf16 v) { return __bfloat162float(v); }

@@ -22,9 +22,6 @@
 
 namespace lory {
 
-__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void pdl_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-
 struct DecodeParams {
   const bf16 *wa, *wb;  // blocked weights [R, K] of every segment: Wbar1, Wbar3 (gate) or Wbar2
   const bf16* x;        // [S, n, K] tokens: x or H

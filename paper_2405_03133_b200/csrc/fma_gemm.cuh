@@ -109,6 +109,8 @@ __global__ void __launch_bounds__(128 * KG, 3) fma_gemm_kernel(const __grid_cons
   while (ji + 1 < p.jobs && tile >= p.job[ji].tile_end) ++ji;
   const FmaJob& J = p.job[ji];
   tile -= ji ? p.job[ji - 1].tile_end : 0;
+  pdl_launch();
+  pdl_wait();
   const int m0 = tile % J.m_tiles * BM, rest = tile / J.m_tiles, n0 = rest % J.n_tiles * TILE_N, g = rest / J.n_tiles;
   const int nkb = (J.K + BK - 1) / BK, total = MODE == FMA_DUALK ? 2 * nkb : nkb;
 

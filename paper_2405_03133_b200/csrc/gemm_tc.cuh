@@ -54,12 +54,10 @@ struct TcTile {
   static constexpr int B_BYTES = (BN / CTAS) * BK * 2;
   static constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
   static constexpr int OUT_BYTES = 128 * 128;  // one 128-row x 64-column bf16 staging tile
-  static constexpr int NARROW_STAGES = (227 * 1024 - 512 - 2 * OUT_BYTES - 1024) / STAGE_BYTES;
   // the SwiGLU-backward epilogue trades pipeline stages for two input staging tiles (G, U)
-  static constexpr int STAGES = (AROWS < 128) ? (NARROW_STAGES > 16 ? 16 : NARROW_STAGES)
-                                : (CTAS == 2) ? ((EPI == EPI_DSWIGLU) ? 5 : 6)
-                                              : ((EPI == EPI_DSWIGLU) ? 3 : ((BN == 256) ? 4 : 6));
   static constexpr int IN_BYTES = (EPI == EPI_DSWIGLU) ? 2 * OUT_BYTES : 0;
+  static constexpr int FIT = (227 * 1024 - 512 - 2 * OUT_BYTES - IN_BYTES - 1024) / STAGE_BYTES;
+  static constexpr int STAGES = (AROWS < 128) ? (FIT > 16 ? 16 : FIT) : (FIT > 8 ? 8 : FIT);
   static constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 2 * OUT_BYTES + IN_BYTES + 1024;  // + alignment slack
 };
 
@@ -159,7 +157,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__
   constexpr int STAGES = Tile::STAGES;
   constexpr int TILE_N = (MODE == MODE_DUALB) ? BN / 2 : BN;  // output columns per tile
   static_assert(!(MODE == MODE_DUALB && B_MN), "MODE_DUALB expects K-major B");
-  static_assert(EPI != EPI_SWIGLU || (MODE == MODE_DUALB && BN == 256), "SwiGLU epilogue needs [G|U] tiles");
+  static_assert(EPI != EPI_SWIGLU || MODE == MODE_DUALB, "SwiGLU epilogue needs [G|U] tiles");
 
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
@@ -206,6 +204,8 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__
   if (PAIR) ptx::cluster_sync();  // both CTAs' barriers exist before either signals the other
   ptx::tc_fence_after_sync();
   const uint32_t tmem_base = tmem_base_smem;
+  pdl_launch();
+  pdl_wait();   // the operands are complete, and nothing in front still reads what this kernel writes
 
   if (warp == 0) {
     // ------------------------------ TMA producer ------------------------------

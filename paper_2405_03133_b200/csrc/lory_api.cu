@@ -305,7 +305,9 @@ static int forward_impl(const lory_dims& D, const Layout& Lo, const T* x, const 
                         const T* w3, T* y, float* route_w, float* route_p, const float* injected_w, char* ws,
                         cudaStream_t st, const T* residual = nullptr) {
   const int N = D.L / D.T, S = D.B * N;
-  if (!(use_tc(D) && tc_clears_status(D))) LORY_CUDA_OK(cudaMemsetAsync(ws + Lo.status, 0, 256, st));
+  // the routing step and the decode kernels clear the status word themselves
+  const bool routes = !(D.flags & LORY_FLAG_REUSE_MERGED) && !injected_w;
+  if (!routes && !(use_tc(D) && tc_clears_status(D))) LORY_CUDA_OK(cudaMemsetAsync(ws + Lo.status, 0, 256, st));
   float* w = (float*)(ws + Lo.w);
   bool w_is_split = false;
   if (D.flags & LORY_FLAG_REUSE_MERGED) {
@@ -318,6 +320,7 @@ static int forward_impl(const lory_dims& D, const Layout& Lo, const T* x, const 
     ProfScope ps("pool_router", st);
     RouteExtra extra;
     extra.w_copy = route_w;
+    extra.status = (uint32_t*)(ws + Lo.status);
     if (D.dtype == LORY_BF16 && use_tc(D)) {
       tc_split_tables(D, Lo, ws, &extra.hi, &extra.lo, &extra.comb, &extra.Epad, &extra.frag);
       w_is_split = true;

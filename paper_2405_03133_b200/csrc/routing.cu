@@ -2,12 +2,16 @@
 // (Eq. 3 and Algorithm 1 of the Lory paper).  All arithmetic in fp32.
 #include "routing.cuh"
 
+#include <cooperative_groups.h>
+
 namespace lory {
 
 // ---------------------------------------------------------------------------------------
 // h_bar[s, :] = (1/T) sum_t x[s*T + t, :]
-// grid (S, ceil(d / (32*VEC))), block 256 = 8 warps; warp w sums rows w, w+8, ...;
-// a lane owns VEC consecutive columns (one 16-byte load per row).
+// HBM-bound (x once).  A block of 8 warps sums a run of a segment's tokens for 32 * VEC columns, warp w rows w, w+8, ...
+// of it, a lane VEC consecutive columns (one 16-byte load per row).  Where there are too few segments to fill the GPU,
+// the blocks of a cluster (up to 8) share a segment's tokens and the first adds their sums through distributed shared
+// memory, in a fixed order (2 segments of 1000 tokens, d = 1024: 30 -> 4 us; with enough segments clusters only cost).
 // ---------------------------------------------------------------------------------------
 template <typename T>
 struct Vec16;
@@ -35,21 +39,26 @@ struct Vec16<bf16> {
 
 template <typename T>
 __global__ void __launch_bounds__(256) pool_kernel(const T* __restrict__ x, float* __restrict__ h_bar,
-                                                    int Tseg, int d) {
+                                                    int Tseg, int d, int parts, uint32_t* status) {
   constexpr int VEC = Vec16<T>::N;
-  const int s = blockIdx.x;
+  const int s = blockIdx.x / parts, part = blockIdx.x - s * parts;   // part = rank in the cluster
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int col = (blockIdx.y * 32 + lane) * VEC;
   __shared__ float red[8][32 * VEC];
+  __shared__ float xch[8][32 * VEC];   // the first block's: one row per block of the cluster
+  pdl_launch();
+  pdl_wait();
+  if (status && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x < 64) status[threadIdx.x] = 0;
+  const int run = (Tseg + parts - 1) / parts, t_end = min(Tseg, (part + 1) * run);
   float acc[VEC];
 #pragma unroll
   for (int i = 0; i < VEC; ++i) acc[i] = 0.f;
   const bool vec_ok = (col + VEC <= d) && (d % VEC == 0);
   const T* base = x + (size_t)s * Tseg * d;
+  int t = part * run + warp;
   if (vec_ok) {
     // four independent 16-byte loads in flight per lane
-    int t = warp;
-    for (; t + 24 < Tseg; t += 32) {
+    for (; t + 24 < t_end; t += 32) {
       float v0[VEC], v1[VEC], v2[VEC], v3[VEC];
       Vec16<T>::load(base + (size_t)t * d + col, v0);
       Vec16<T>::load(base + (size_t)(t + 8) * d + col, v1);
@@ -58,14 +67,15 @@ __global__ void __launch_bounds__(256) pool_kernel(const T* __restrict__ x, floa
 #pragma unroll
       for (int i = 0; i < VEC; ++i) acc[i] += (v0[i] + v1[i]) + (v2[i] + v3[i]);
     }
-    for (; t < Tseg; t += 8) {
+#pragma unroll 4
+    for (; t < t_end; t += 8) {
       float v[VEC];
       Vec16<T>::load(base + (size_t)t * d + col, v);
 #pragma unroll
       for (int i = 0; i < VEC; ++i) acc[i] += v[i];
     }
   } else {
-    for (int t = warp; t < Tseg; t += 8) {
+    for (; t < t_end; t += 8) {
       const T* row = base + (size_t)t * d;
 #pragma unroll
       for (int i = 0; i < VEC; ++i)
@@ -75,13 +85,23 @@ __global__ void __launch_bounds__(256) pool_kernel(const T* __restrict__ x, floa
 #pragma unroll
   for (int i = 0; i < VEC; ++i) red[warp][lane * VEC + i] = acc[i];
   __syncthreads();
-  for (int c = threadIdx.x; c < 32 * VEC; c += 256) {
-    float sum = 0.f;
+  const int c = threadIdx.x, gc = blockIdx.y * 32 * VEC + c;
+  float sum = 0.f;
+  if (c < 32 * VEC) {
 #pragma unroll
     for (int w = 0; w < 8; ++w) sum += red[w][c];
-    int gc = blockIdx.y * 32 * VEC + c;
-    if (gc < d) h_bar[(size_t)s * d + gc] = sum / (float)Tseg;
   }
+  if (parts > 1) {
+    namespace cg = cooperative_groups;
+    cg::cluster_group cluster = cg::this_cluster();
+    if (c < 32 * VEC) *cluster.map_shared_rank(&xch[part][c], 0) = sum;
+    cluster.sync();
+    if (part > 0) return;
+    sum = 0.f;
+    if (c < 32 * VEC)
+      for (int q = 0; q < parts; ++q) sum += xch[q][c];
+  }
+  if (c < 32 * VEC && gc < d) h_bar[(size_t)s * d + gc] = sum / (float)Tseg;
 }
 
 // ---------------------------------------------------------------------------------------
@@ -135,11 +155,14 @@ __global__ void __launch_bounds__(1024) router_kernel(const float* __restrict__ 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const float* h = h_bar + (size_t)s * d;
   const int nwarps = blockDim.x >> 5;
+  pdl_launch();
+  pdl_wait();
   for (int e = warp; e < E; e += nwarps) {
     const T* wr = w_r + (size_t)e * d;
     float acc = 0.f;
     constexpr int VEC = Vec16<T>::N;
     if (d % VEC == 0) {
+#pragma unroll 4
       for (int j = lane * VEC; j < d; j += 32 * VEC) {
         float wv[VEC];
         Vec16<T>::load(wr + j, wv);
@@ -194,71 +217,80 @@ __global__ void __launch_bounds__(1024) router_kernel(const float* __restrict__ 
 // Backward of the router path.
 // ---------------------------------------------------------------------------------------
 // dw[s,:] = sum of the partial slabs; dz_s = p_s * (dp_s - <dp_s, p_s>) with dp_{b,n} = dw_{b,n+1} (0 for the
-// last segment); dh_bar_s = W_r^T dz_s.  One block per segment; the block sums the slab rows it needs itself
-// (its own row for the dw output, the next segment's row for dp).
+// last segment); dh_bar_s = W_r^T dz_s.  One block per segment.  Latency-bound: the block's threads are spread over the
+// 2 E values it needs (its own row for the dw output and, next to it in a slab, the next segment's for dp) and over the
+// slabs, with eight loads in flight each; a chain of one load per slab and warp took most of the 16 us this kernel had
+// (8 segments, 8 experts, 444 slabs: now 6).
+static const int kRouterBwdThreads = 512;
 template <typename T>
-__global__ void __launch_bounds__(256) router_bwd_kernel(const float* __restrict__ partial, int n_slabs,
-                                                         const float* __restrict__ p,
-                                                         const T* __restrict__ w_r, float* __restrict__ dw,
-                                                         float* __restrict__ d_route_w, float* __restrict__ dz,
-                                                         float* __restrict__ dh_bar, int S, int N, int d, int E,
-                                                         int prefix) {
-  __shared__ float red[8][128];
-  extern __shared__ float sm[];  // dp[E], dz[E]
-  float* dp_sm = sm;
-  float* dz_sm = sm + E;
-  const int s = blockIdx.x;
-  const int n = s % N;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+__global__ void __launch_bounds__(kRouterBwdThreads)
+router_bwd_kernel(const float* __restrict__ partial, int n_slabs, const float* __restrict__ p, const T* __restrict__ w_r,
+                  float* __restrict__ dw, float* __restrict__ d_route_w, float* __restrict__ dz,
+                  float* __restrict__ dh_bar, int S, int N, int d, int E, int prefix) {
+  constexpr int NT = kRouterBwdThreads, VEC = Vec16<T>::N;
+  __shared__ __align__(16) float red[3 * 128 * VEC > NT ? 3 * 128 * VEC : NT];
+  extern __shared__ float sm[];  // rows[2 E], dz[E]
+  float* dw_sm = sm;
+  float* dp_sm = sm + E;
+  float* dz_sm = sm + 2 * E;
+  const int s = blockIdx.x, n = s % N, tid = threadIdx.x;
+  const int lane = tid & 31, warp = tid >> 5;
   const size_t SE = (size_t)S * E;
-  // Sums one [E] row over the slabs, 128 experts at a time (every thread of the block calls this).
-  // mode 0: the row is this segment's dw (written out); 1: dp = row; 2: dp += row.
-  auto reduce_row = [&](size_t row, int mode) {
-    for (int e0 = 0; e0 < E; e0 += 128) {
-      for (int e = e0 + lane; e < min(E, e0 + 128); e += 32) {
-        // four independent partial sums: the loads of four slabs are in flight together
-        float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
-        const float* src = partial + row * E + e;
-        int c = warp;
-        for (; c + 24 < n_slabs; c += 32) {
-          a0 += src[(size_t)c * SE];
-          a1 += src[(size_t)(c + 8) * SE];
-          a2 += src[(size_t)(c + 16) * SE];
-          a3 += src[(size_t)(c + 24) * SE];
-        }
-        for (; c < n_slabs; c += 8) a0 += src[(size_t)c * SE];
-        red[warp][e - e0] = (a0 + a1) + (a2 + a3);
-      }
-      __syncthreads();
-      for (int e = e0 + threadIdx.x; e < min(E, e0 + 128); e += 256) {
-        float t = 0.f;
+  pdl_launch();
+  pdl_wait();
+  // out[c] (+)= sum over the slabs and over `rows` consecutive segments of the values of segment `row` on, c < width
+  auto reduce = [&](float* out, size_t row, int width, int rows, bool add) {
+    int span = 32;
+    while (span < width && span < NT) span <<= 1;
+    const int groups = NT / span, g = tid / span, total = n_slabs * rows;
+    for (int c0 = 0; c0 < width; c0 += span) {
+      const int c = c0 + (tid & (span - 1));
+      float acc = 0.f;
+      if (c < width) {
+        const float* src = partial + row * E + c;
+        int q = g;
+        for (; q + 7 * groups < total; q += 8 * groups) {
+          float v[8];
 #pragma unroll
-        for (int w = 0; w < 8; ++w) t += red[w][e - e0];
-        if (mode == 0) {
-          dw[row * E + e] = t;
-          if (d_route_w) d_route_w[row * E + e] = t;
-        } else if (mode == 1) {
-          dp_sm[e] = t;
-        } else {
-          dp_sm[e] += t;
+          for (int i = 0; i < 8; ++i) {
+            const int k = q + i * groups, m = rows == 1 ? 0 : k / n_slabs;
+            v[i] = src[(size_t)(k - m * n_slabs) * SE + (size_t)m * E];
+          }
+          acc += ((v[0] + v[1]) + (v[2] + v[3])) + ((v[4] + v[5]) + (v[6] + v[7]));
         }
+#pragma unroll 4
+        for (; q < total; q += groups) {
+          const int m = rows == 1 ? 0 : q / n_slabs;
+          acc += src[(size_t)(q - m * n_slabs) * SE + (size_t)m * E];
+        }
+      }
+      red[tid] = acc;
+      __syncthreads();
+      if (tid < span && c < width) {
+        float v = 0.f;
+        for (int k = 0; k < groups; ++k) v += red[k * span + tid];
+        out[c] = add ? out[c] + v : v;
       }
       __syncthreads();
     }
   };
-  reduce_row((size_t)s, 0);
-  for (int e = threadIdx.x; e < E; e += 256) dp_sm[e] = 0.f;
-  __syncthreads();
+  const bool prefix_mode = (prefix & 1) != 0, first_grad = (prefix & 2) != 0;
   // gradient reaching p_s: from the next segment's weights, or (prefix routing) from segments 1..N-1 if s is the
   // first segment of its sequence; the first segment's own use of p_s carries no gradient (stop-gradient)
-  const bool prefix_mode = (prefix & 1) != 0, first_grad = (prefix & 2) != 0;
-  if (!prefix_mode) {
-    if (n < N - 1) reduce_row((size_t)s + 1, 1);
-  } else if (n == 0) {
-    for (int m = 1; m < N; ++m) reduce_row((size_t)s + m, 2);
+  const bool next = !prefix_mode && n < N - 1;
+  reduce(dw_sm, (size_t)s, next ? 2 * E : E, 1, false);
+  if (!next) {
+    for (int e = tid; e < E; e += NT) dp_sm[e] = 0.f;
+    __syncthreads();
+    if (prefix_mode && n == 0 && N > 1) reduce(dp_sm, (size_t)s + 1, E, N - 1, true);
   }
-  // without the stop-gradient the first segment's own weights also feed p_s
-  if (first_grad && n == 0) reduce_row((size_t)s, 2);
+  for (int e = tid; e < E; e += NT) {
+    const float v = dw_sm[e];
+    dw[(size_t)s * E + e] = v;
+    if (d_route_w) d_route_w[(size_t)s * E + e] = v;
+    if (first_grad && n == 0) dp_sm[e] += v;   // no stop-gradient: the first segment's own weights also feed p_s
+  }
+  __syncthreads();
   if (warp == 0) {
     float dot = 0.f;
     for (int e = lane; e < E; e += 32) dot += dp_sm[e] * p[(size_t)s * E + e];
@@ -271,13 +303,11 @@ __global__ void __launch_bounds__(256) router_bwd_kernel(const float* __restrict
     }
   }
   __syncthreads();
-  // dh_bar_s = W_r^T dz_s.  A thread takes VEC consecutive columns (one 16-byte load per expert row) and one
-  // half of the experts; the two halves of the block meet in shared memory.  All loads of a thread are independent.
-  constexpr int VEC = Vec16<T>::N;
+  // dh_bar_s = W_r^T dz_s.  A thread takes VEC consecutive columns (one 16-byte load per expert row) and a quarter of the
+  // experts; the quarters meet in shared memory.  All loads of a thread are independent.
   if (d % VEC == 0) {
-    float* xch = &red[0][0];  // 128 threads x VEC <= 1024 floats
-    const int nvec = d / VEC, half = threadIdx.x >> 7, vt = threadIdx.x & 127;
-    const int eh = (E + 1) / 2, e_begin = half * eh, e_end = min(E, e_begin + eh);
+    const int nvec = d / VEC, quarter = tid >> 7, vt = tid & 127;
+    const int eq = (E + 3) / 4, e_begin = quarter * eq, e_end = min(E, e_begin + eq);
     for (int v0 = 0; v0 < nvec; v0 += 128) {
       const int v = v0 + vt;
       float acc[VEC];
@@ -293,23 +323,22 @@ __global__ void __launch_bounds__(256) router_bwd_kernel(const float* __restrict
           for (int i = 0; i < VEC; ++i) acc[i] += z * wv[i];
         }
       }
-      if (half == 1) {
+      if (quarter > 0) {
 #pragma unroll
-        for (int i = 0; i < VEC; ++i) xch[i * 128 + vt] = acc[i];
+        for (int i = 0; i < VEC; ++i) red[((quarter - 1) * VEC + i) * 128 + vt] = acc[i];
       }
       __syncthreads();
-      if (half == 0 && v < nvec) {
+      if (quarter == 0 && v < nvec) {
 #pragma unroll
-        for (int i = 0; i < VEC; i += 4) {
-          float4 o = make_float4(acc[i] + xch[i * 128 + vt], acc[i + 1] + xch[(i + 1) * 128 + vt],
-                                 acc[i + 2] + xch[(i + 2) * 128 + vt], acc[i + 3] + xch[(i + 3) * 128 + vt]);
-          *reinterpret_cast<float4*>(dh_bar + (size_t)s * d + (size_t)v * VEC + i) = o;
-        }
+        for (int i = 0; i < VEC; ++i) acc[i] += red[i * 128 + vt] + red[(VEC + i) * 128 + vt] + red[(2 * VEC + i) * 128 + vt];
+#pragma unroll
+        for (int i = 0; i < VEC; i += 4)
+          *reinterpret_cast<float4*>(dh_bar + (size_t)s * d + (size_t)v * VEC + i) = make_float4(acc[i], acc[i + 1], acc[i + 2], acc[i + 3]);
       }
       __syncthreads();
     }
   } else {
-    for (int j = threadIdx.x; j < d; j += blockDim.x) {
+    for (int j = tid; j < d; j += NT) {
       float a0 = 0.f;
       for (int e = 0; e < E; ++e) a0 += dz_sm[e] * to_f32(w_r[(size_t)e * d + j]);
       dh_bar[(size_t)s * d + j] = a0;
@@ -328,6 +357,8 @@ __global__ void __launch_bounds__(512) dwr_kernel(const float* __restrict__ dz, 
   const int j = blockIdx.x * 64 + jj, e0 = blockIdx.y * 4;
   const int run = (S + 7) / 8;
   const int s_begin = part * run, s_end = min(S, s_begin + run);
+  pdl_launch();
+  pdl_wait();
   float a[4] = {0.f, 0.f, 0.f, 0.f};
   if (j < d) {
 #pragma unroll 4
@@ -361,13 +392,15 @@ int launch_pool_router(const T* x, const T* w_r, float* h_bar, float* p_ws, floa
                        int B, int N, int Tseg, int d, int E, int prefix, cudaStream_t st, RouteExtra extra) {
   const int S = B * N;
   constexpr int VEC = Vec16<T>::N;
-  dim3 grid(S, (unsigned)ceil_div(d, 32 * VEC));
-  pool_kernel<T><<<grid, 256, 0, st>>>(x, h_bar, Tseg, d);
-  LORY_AFTER_LAUNCH();
+  const long blocks = S * ceil_div(d, 32 * VEC);
+  // a cluster per segment until there are two blocks per SM, as long as each block has 32 rows
+  int parts = 1;
+  while (parts < 8 && blocks * parts < 296 && Tseg >= 64 * parts) parts *= 2;
+  LORY_TRY(launch_overlapped(pool_kernel<T>, dim3((unsigned)(S * parts), (unsigned)ceil_div(d, 32 * VEC)), 256, 0, st, parts, x,
+                             h_bar, Tseg, d, parts, extra.status));
   const int router_threads = E >= 32 ? 1024 : (E > 8 ? 32 * E : 256);  // one warp per expert, 8 to 32 warps
-  router_kernel<T><<<S, router_threads, E * sizeof(float), st>>>(h_bar, w_r, p_ws, route_p, w_out, N, d, E, prefix, extra);
-  LORY_AFTER_LAUNCH();
-  return LORY_OK;
+  return launch_overlapped(router_kernel<T>, dim3((unsigned)S), router_threads, E * sizeof(float), st, 1, h_bar, w_r, p_ws,
+                           route_p, w_out, N, d, E, prefix, extra);
 }
 
 template <typename T>
@@ -375,11 +408,12 @@ int launch_router_backward(const float* dw_partial, int n_slabs, const float* p_
                            const T* w_r, float* dw, float* d_route_w, float* dz, float* dh_bar, T* dw_r,
                            int B, int N, int d, int E, int prefix, cudaStream_t st) {
   const int S = B * N;
-  router_bwd_kernel<T><<<S, 256, 2 * E * sizeof(float), st>>>(dw_partial, n_slabs, p_ws, w_r, dw, d_route_w, dz, dh_bar, S, N, d, E, prefix);
-  LORY_AFTER_LAUNCH();
-  dwr_kernel<T><<<dim3((unsigned)ceil_div(d, 64), (unsigned)ceil_div(E, 4)), 512, 0, st>>>(dz, h_bar, dw_r, S, d, E, (prefix & 4) ? 1 : 0);
-  LORY_AFTER_LAUNCH();
-  return LORY_OK;
+  const size_t smem = 3 * (size_t)E * sizeof(float);   // up to 48 KB beside the static 12 KB
+  if (smem > 32 * 1024) LORY_CUDA_OK(cudaFuncSetAttribute(router_bwd_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, 48 * 1024));
+  LORY_TRY(launch_overlapped(router_bwd_kernel<T>, dim3((unsigned)S), kRouterBwdThreads, smem, st, 1, dw_partial, n_slabs, p_ws,
+                             w_r, dw, d_route_w, dz, dh_bar, S, N, d, E, prefix));
+  return launch_overlapped(dwr_kernel<T>, dim3((unsigned)ceil_div(d, 64), (unsigned)ceil_div(E, 4)), 512, 0, st, 1, dz, h_bar,
+                           dw_r, S, d, E, (prefix & 4) ? 1 : 0);
 }
 
 // one thread per expert; the S weights of an expert are E floats apart

@@ -18,6 +18,7 @@ struct RouteExtra {
   bf16* comb = nullptr;
   int Epad = 0;
   bf16* frag = nullptr;
+  uint32_t* status = nullptr;  // 64 words the pooling kernel clears
 };
 template <typename T>
 int launch_pool_router(const T* x, const T* w_r, float* h_bar, float* p_ws, float* route_p, float* w_out,

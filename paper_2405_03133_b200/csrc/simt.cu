@@ -130,18 +130,16 @@ static int fma_launch(FmaArgs a, int groups, cudaStream_t st) {
     vec = vec && j.lda % 4 == 0 && j.ldb % 4 == 0 && j.a_g % 4 == 0 && j.b_g % 4 == 0 && in % (4 * sizeof(T)) == 0 &&
           (A_K ? j.K : j.M) % 4 == 0 && (B_K ? j.K : j.N) % 4 == 0;
   }
-  auto pick = [&](auto v) {
+  const dim3 grid((unsigned)tiles);
+  auto pick = [&](auto v) -> int {
     constexpr bool V = decltype(v)::value;
     const bool two = bm == 32 || tiles < 3L * sms;
-    if (bm == 128) fma_gemm_kernel<T, A_K, B_K, MODE, EPI, 128, 1, V><<<(unsigned)tiles, 128, 0, st>>>(a);
-    else if (bm == 64 && two) fma_gemm_kernel<T, A_K, B_K, MODE, EPI, 64, 2, V><<<(unsigned)tiles, 256, 0, st>>>(a);
-    else if (bm == 64) fma_gemm_kernel<T, A_K, B_K, MODE, EPI, 64, 1, V><<<(unsigned)tiles, 128, 0, st>>>(a);
-    else fma_gemm_kernel<T, A_K, B_K, MODE, EPI, 32, 2, V><<<(unsigned)tiles, 256, 0, st>>>(a);
+    if (bm == 128) return launch_kernel(false, fma_gemm_kernel<T, A_K, B_K, MODE, EPI, 128, 1, V>, grid, 128, 0, st, 1, a);
+    if (bm == 64 && two) return launch_kernel(false, fma_gemm_kernel<T, A_K, B_K, MODE, EPI, 64, 2, V>, grid, 256, 0, st, 1, a);
+    if (bm == 64) return launch_kernel(false, fma_gemm_kernel<T, A_K, B_K, MODE, EPI, 64, 1, V>, grid, 128, 0, st, 1, a);
+    return launch_kernel(false, fma_gemm_kernel<T, A_K, B_K, MODE, EPI, 32, 2, V>, grid, 256, 0, st, 1, a);
   };
-  if (vec) pick(std::true_type());
-  else pick(std::false_type());
-  LORY_AFTER_LAUNCH();
-  return LORY_OK;
+  return vec ? pick(std::true_type()) : pick(std::false_type());
 }
 static FmaArgs one_job(const FmaJob& j) {
   FmaArgs a = {};
@@ -179,6 +177,8 @@ __global__ void __launch_bounds__(128) fma_merge_kernel(const __grid_constant__ 
   constexpr int SC = 16;
   __shared__ __align__(16) float s_w[32][SC];  // [expert][segment of the chunk]
   const int k = blockIdx.y;
+  pdl_launch();
+  pdl_wait();
   const long i0 = ((long)blockIdx.x * 128 + threadIdx.x) * 4;
   const int left = i0 < p.n ? (int)min(4L, p.n - i0) : 0;
   const bool vec = (p.n & 3) == 0 && (((uintptr_t)p.w[k] | (uintptr_t)p.wbar[k]) & (4 * sizeof(T) - 1)) == 0;
@@ -235,6 +235,8 @@ __global__ void __launch_bounds__(256) fma_adjoint_kernel(const __grid_constant_
   float* s_dw = s_w + kFmaSegs * EMAX;         // [S][E]
   const int tid = threadIdx.x, ks = tid & 3, sg = (tid >> 2) & 7, eg = tid >> 5;
   for (int i = tid; i < p.S * p.E; i += 256) s_dw[i] = 0.f;
+  pdl_launch();
+  pdl_wait();
   const int per = (int)((p.n + kFmaTile - 1) / kFmaTile), chunks = (p.S + kFmaSegs - 1) / kFmaSegs;
   // One step = one chunk of segments of one tile.  The next step's values are on their way in registers (ve, vd) while
   // this one is worked on: 198 -> 128 us at S = 18, E = 6, n = 670 000.
@@ -344,17 +346,13 @@ int fma_adjoint_slabs(long n) {
 }
 template <typename T>
 int launch_fma_merge(const FmaMerge<T>& p, cudaStream_t st) {
-  fma_merge_kernel<T><<<dim3((unsigned)ceil_div(p.n, 512), 3), 128, 0, st>>>(p);
-  LORY_AFTER_LAUNCH();
-  return LORY_OK;
+  return launch_kernel(false, fma_merge_kernel<T>, dim3((unsigned)ceil_div(p.n, 512), 3), 128, 0, st, 1, p);
 }
 template <typename T, int EMAX>
 static int launch_fma_adjoint_t(const FmaMerge<T>& p, cudaStream_t st) {
   const size_t smem = fma_adjoint_smem(p.S, p.E, EMAX);
   LORY_CUDA_OK(cudaFuncSetAttribute(fma_adjoint_kernel<T, EMAX>, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024));
-  fma_adjoint_kernel<T, EMAX><<<fma_adjoint_slabs(p.n), 256, smem, st>>>(p);
-  LORY_AFTER_LAUNCH();
-  return LORY_OK;
+  return launch_kernel(false, fma_adjoint_kernel<T, EMAX>, dim3((unsigned)fma_adjoint_slabs(p.n)), 256, smem, st, 1, p);
 }
 template <typename T>
 int launch_fma_adjoint(const FmaMerge<T>& p, cudaStream_t st) {

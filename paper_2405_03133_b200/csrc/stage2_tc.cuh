@@ -136,6 +136,8 @@ stage2_kernel(const __grid_constant__ Stage2Maps maps, const Stage2Params p) {
   ptx::tc_fence_after_sync();
   const uint32_t tmem_base = tmem_base_smem;
   const uint32_t tmem_d2 = tmem_base + NACC * ACC_COLS;
+  pdl_launch();
+  pdl_wait();
 
   // second product of one stage: dw [s, e] += dWbar [s, p] . W^T [p, e]   (one accumulator per group of 128 segments,
   // resident in TMEM for the whole kernel; with fewer than 128 segments in the box the rows past them hold whatever

@@ -109,6 +109,8 @@ __global__ void __launch_bounds__(32 * NW) merge_stream_kernel(const __grid_cons
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
   const unsigned total = p.piece_end[2];
   const unsigned base = (blockIdx.x * NW + warp) * U;
+  pdl_launch();
+  pdl_wait();
   if (base >= total) return;
   uint4 v[U][KT][4];
   bf16* out[U];
@@ -223,6 +225,8 @@ adjoint_stream_kernel(const __grid_constant__ StreamAdjointParams p) {
   uint4* s_a = s_ring + NW * STG * A::STAGE / 16;            // [16 experts][16 segments][hi, lo][lane]
   float* s_dw = reinterpret_cast<float*>(s_a + ET * ST * 64);  // [16 ST][16 ET]
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+  pdl_launch();
+  pdl_wait();
   for (int i = threadIdx.x; i < ET * ST * 32; i += NT) {
     const int ln = i & 31, m = (i >> 5) % ST, em = (i >> 5) / ST;
     a_fragment(ln, [&](int row, int col) {

@@ -162,25 +162,7 @@ static int launch_tc(const char* label, const CUtensorMap& a0, const CUtensorMap
   const CUtensorMap& me0 = e0 ? *e0 : c0;
   const CUtensorMap& me1 = e1 ? *e1 : c0;
   ProfScope ps(label, st);
-  if (CTAS == 1) {
-    kern<<<grid, 192, Tile::SMEM_BYTES, st>>>(a0, a1, b0, b1, c0, c1, c2, me0, me1, p);
-  } else {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(grid);
-    cfg.blockDim = dim3(192);
-    cfg.dynamicSmemBytes = Tile::SMEM_BYTES;
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = 2;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    LORY_CUDA_OK(cudaLaunchKernelEx(&cfg, kern, a0, a1, b0, b1, c0, c1, c2, me0, me1, p));
-  }
-  LORY_AFTER_LAUNCH();
-  return LORY_OK;
+  return launch_overlapped(kern, dim3((unsigned)grid), 192, Tile::SMEM_BYTES, st, CTAS, a0, a1, b0, b1, c0, c1, c2, me0, me1, p);
 }
 
 // One per-segment weight gradient C_g = A_g^T B_g (K = T): the resident-operand kernel for CTA-pair tiles with short
@@ -202,23 +184,9 @@ static int launch_wgrad(const CUtensorMap& a, const CUtensorMap& b, const CUtens
     LORY_TRY(allow_dynamic_smem(wgrad_kernel<false>, WgradTile::SMEM_BYTES, attr_set[0]));
     LORY_TRY(allow_dynamic_smem(wgrad_kernel<true>, WgradTile::SMEM_BYTES, attr_set[1]));
     const int slots = sm_count() / 2;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(2 * (unsigned)(strips < slots ? strips : slots));
-    cfg.blockDim = dim3(192);
-    cfg.dynamicSmemBytes = WgradTile::SMEM_BYTES;
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = 2;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    const dim3 grid(2 * (unsigned)(strips < slots ? strips : slots));
     ProfScope ps("wgrad", st);
-    if (res_a) LORY_CUDA_OK(cudaLaunchKernelEx(&cfg, wgrad_kernel<true>, a, b, c, p));
-    else LORY_CUDA_OK(cudaLaunchKernelEx(&cfg, wgrad_kernel<false>, a, b, c, p));
-    LORY_AFTER_LAUNCH();
-    return LORY_OK;
+    return launch_overlapped(res_a ? wgrad_kernel<true> : wgrad_kernel<false>, grid, 192, WgradTile::SMEM_BYTES, st, 2, a, b, c, p);
   }
   TcGemmParams p = {};
   p.groups = groups; p.K = K; p.M = M; p.N = N; p.status = status;
@@ -444,9 +412,7 @@ static int check_vector_aligned(const void* const* ptrs, int n) {
 template <int KT, int U, int NW>
 static int launch_merge_t(const StreamMergeParams& p, cudaStream_t st) {
   ProfScope ps("merge", st);
-  merge_stream_kernel<KT, U, NW><<<(unsigned)ceil_div(p.piece_end[2], NW * U), 32 * NW, 0, st>>>(p);
-  LORY_AFTER_LAUNCH();
-  return LORY_OK;
+  return launch_kernel(false, merge_stream_kernel<KT, U, NW>, dim3((unsigned)ceil_div(p.piece_end[2], NW * U)), 32 * NW, 0, st, 1, p);
 }
 // Wbar_k (blocked) = (w_hi + w_lo) . W_k for the three matrices in one launch      (Eq. 2)
 static int launch_merge(const lory_dims& D, const WsPtrs& q, const bf16* const src[3], bf16* const dst[3],
@@ -502,9 +468,7 @@ static int launch_adjoint_stream(const lory_dims& D, const WsPtrs& q, const AdjP
       p.stages = A::STG >= 3 && A::CTAS * A::NW * (p.S + 2 * p.E) * 128 < 70 * 1024 ? 3 : 2;
       LORY_TRY(allow_dynamic_smem(kern, A::SMEM, done));
       ProfScope ps("stage2", st);
-      kern<<<ctas, 32 * A::NW, A::SMEM, st>>>(p);
-      LORY_AFTER_LAUNCH();
-      return LORY_OK;
+      return launch_overlapped(kern, dim3((unsigned)ctas), 32 * A::NW, A::SMEM, st, 1, p);
     };
     static bool done[2][kMaxDevices];
     if (acc) return launch(adjoint_stream_kernel<S::S16, S::E16, true>, AdjointStream<S::S16, S::E16, true>(), done[1]);
@@ -584,9 +548,8 @@ static int launch_stage2(const lory_dims& D, const WsPtrs& q, const AdjPiece pc[
     p.S = S - base < 256 ? S - base : 256;
     p.s_tiles = (p.S + 127) / 128;
     ProfScope ps("stage2", st);
-    if (base > 0 || (D.flags & LORY_FLAG_ACCUMULATE_GRADS)) stage2_kernel<true><<<grid, 224, smem, st>>>(maps, p);
-    else stage2_kernel<false><<<grid, 224, smem, st>>>(maps, p);
-    LORY_AFTER_LAUNCH();
+    const bool add = base > 0 || (D.flags & LORY_FLAG_ACCUMULATE_GRADS);
+    LORY_TRY(launch_overlapped(add ? stage2_kernel<true> : stage2_kernel<false>, dim3((unsigned)grid), 224, smem, st, 1, maps, p));
   }
   return LORY_OK;
 }
@@ -601,30 +564,13 @@ void tc_split_tables(const lory_dims& D, const Layout& Lo, char* ws, bf16** hi, 
   *frag = q.w_frag;
 }
 
-// Launch attribute of programmatic dependent launch: the kernel may start while its predecessor runs (it waits itself).
-template <typename K, typename P>
-static int launch_pdl(K kern, dim3 grid, int threads, int smem, const P& p, cudaStream_t st) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = grid;
-  cfg.blockDim = dim3(threads);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  LORY_CUDA_OK(cudaLaunchKernelEx(&cfg, kern, p));
-  LORY_AFTER_LAUNCH();
-  return LORY_OK;
-}
 template <int MODE, int NT, int MT>
 static int launch_decode_t(const DecodeParams& p, cudaStream_t st) {
   using D = Decode<MODE, NT, MT>;
   static bool attr_set[kMaxDevices];
   LORY_TRY(allow_dynamic_smem(decode_kernel<MODE, NT, MT>, D::SMEM, attr_set));
   const long tiles = ceil_div(p.R, D::TR) * p.S, cap = (long)D::CTAS * sm_count();
-  return launch_pdl(decode_kernel<MODE, NT, MT>, dim3((unsigned)(tiles < cap ? tiles : cap)), 256, D::SMEM, p, st);
+  return launch_overlapped(decode_kernel<MODE, NT, MT>, dim3((unsigned)(tiles < cap ? tiles : cap)), 256, D::SMEM, st, 1, p);
 }
 // Two weight tiles at a time from 17 tokens on, and below where every CTA still gets three such double tiles (32 sequences,
 // 8 tokens, d = 1024: 109 -> 89 us; with two sequences at d = 2048 the coarser split costs more than it saves: 27 -> 30).

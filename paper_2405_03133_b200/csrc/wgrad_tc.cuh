@@ -96,6 +96,8 @@ wgrad_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
   ptx::cluster_sync();  // both CTAs' barriers exist before either signals the other
   ptx::tc_fence_after_sync();
   const uint32_t tmem_base = tmem_base_smem;
+  pdl_launch();
+  pdl_wait();
 
   if (warp == 0) {
     // ------------------------------ TMA producer (one thread in each CTA) ------------------------------
