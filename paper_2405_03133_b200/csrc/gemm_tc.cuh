@@ -43,21 +43,17 @@ struct TcGemmParams {
 
 // CTAS = 2: two CTAs of a cluster share one 256 x BN tile (tcgen05 cta_group::2); each loads its own
 // 128 rows of A and one half of B's BN columns, which cuts the L2 -> shared-memory traffic per flop by a third.
-// AROWS < 128 (groups of at most AROWS rows: a decode step): only AROWS rows of A are loaded per stage, and the
-// shared memory that frees goes into more stages, i.e. more weight bytes in flight per SM.  The MMA still reads 128
-// rows; rows AROWS.. of its A operand are whatever follows in shared memory (inside the CTA's allocation: the output
-// staging follows the last stage), they only reach accumulator rows that are never stored.
-template <int BN, int EPI, int CTAS = 1, int AROWS = 128>
+template <int BN, int EPI, int CTAS = 1>
 struct TcTile {
   static constexpr int BM = 128, BK = 64;
-  static constexpr int A_BYTES = AROWS * BK * 2;
+  static constexpr int A_BYTES = BM * BK * 2;
   static constexpr int B_BYTES = (BN / CTAS) * BK * 2;
   static constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
   static constexpr int OUT_BYTES = 128 * 128;  // one 128-row x 64-column bf16 staging tile
   // the SwiGLU-backward epilogue trades pipeline stages for two input staging tiles (G, U)
   static constexpr int IN_BYTES = (EPI == EPI_DSWIGLU) ? 2 * OUT_BYTES : 0;
   static constexpr int FIT = (227 * 1024 - 512 - 2 * OUT_BYTES - IN_BYTES - 1024) / STAGE_BYTES;
-  static constexpr int STAGES = (AROWS < 128) ? (FIT > 16 ? 16 : FIT) : (FIT > 8 ? 8 : FIT);
+  static constexpr int STAGES = FIT > 8 ? 8 : FIT;
   static constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 2 * OUT_BYTES + IN_BYTES + 1024;  // + alignment slack
 };
 
@@ -141,16 +137,14 @@ __device__ __forceinline__ void warp_stage_and_store(WarpStager& ws, const CUten
   }
   ws.n++;
 }
-template <bool A_MN, bool B_MN, int BN, int MODE, int EPI, bool B_BLK = false, bool C_BLK = false, int CTAS = 1,
-          int AROWS = 128>
+template <bool A_MN, bool B_MN, int BN, int MODE, int EPI, bool B_BLK = false, bool C_BLK = false, int CTAS = 1>
 __global__ void __launch_bounds__(192, 1)
 tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__ CUtensorMap tmA1,
                const __grid_constant__ CUtensorMap tmB0, const __grid_constant__ CUtensorMap tmB1,
                const __grid_constant__ CUtensorMap tmC0, const __grid_constant__ CUtensorMap tmC1,
                const __grid_constant__ CUtensorMap tmC2, const __grid_constant__ CUtensorMap tmE0,
                const __grid_constant__ CUtensorMap tmE1, const TcGemmParams p) {
-  using Tile = TcTile<BN, EPI, CTAS, AROWS>;
-  static_assert(AROWS == 128 || (!A_MN && CTAS == 1 && EPI != EPI_DSWIGLU), "short A tiles: K-major A, single CTA");
+  using Tile = TcTile<BN, EPI, CTAS>;
   constexpr bool PAIR = (CTAS == 2);
   const int rank = PAIR ? (int)ptx::cluster_ctarank() : 0;  // 0 = leader: arms the full barriers, issues the MMAs
   const int wid = blockIdx.x / CTAS, wstride = gridDim.x / CTAS;

@@ -141,20 +141,19 @@ static int allow_dynamic_smem(K kern, int bytes, bool (&done)[kMaxDevices]) {
 
 static const int kMaxSmem = 227 * 1024 - 512;  // dynamic shared memory we may ask for (static use is < 512 B)
 
-template <bool A_MN, bool B_MN, int BN, int MODE, int EPI, bool B_BLK = false, bool C_BLK = false, int CTAS = 1,
-          int AROWS = 128>
+template <bool A_MN, bool B_MN, int BN, int MODE, int EPI, bool B_BLK = false, bool C_BLK = false, int CTAS = 1>
 static int launch_tc(const char* label, const CUtensorMap& a0, const CUtensorMap& a1, const CUtensorMap& b0,
                      const CUtensorMap& b1, const CUtensorMap& c0, const CUtensorMap& c1, const CUtensorMap& c2,
                      TcGemmParams p, cudaStream_t st, const CUtensorMap* e0 = nullptr,
                      const CUtensorMap* e1 = nullptr) {
   constexpr int TILE_N = (MODE == MODE_DUALB) ? BN / 2 : BN;
-  using Tile = TcTile<BN, EPI, CTAS, AROWS>;
+  using Tile = TcTile<BN, EPI, CTAS>;
   p.m_tiles = (int)ceil_div(p.M, 128 * CTAS);
   p.n_tiles = (int)ceil_div(p.N, TILE_N);
   const long tiles = (long)p.m_tiles * p.n_tiles * p.groups;
   if (tiles <= 0) return LORY_OK;
   if (tiles > 0x7fffffffL) return LORY_ERR_SHAPE;
-  auto kern = tc_gemm_kernel<A_MN, B_MN, BN, MODE, EPI, B_BLK, C_BLK, CTAS, AROWS>;
+  auto kern = tc_gemm_kernel<A_MN, B_MN, BN, MODE, EPI, B_BLK, C_BLK, CTAS>;
   static bool attr_set[kMaxDevices];
   LORY_TRY(allow_dynamic_smem(kern, Tile::SMEM_BYTES, attr_set));
   const int slots = sm_count() / CTAS;  // persistent CTAs (or CTA pairs)
@@ -370,8 +369,32 @@ size_t tc_adjoint_ring_elems(const lory_dims& D) {
   return best;
 }
 
-// CTA pairs (256-row tiles) pay off when a segment fills them.
-static bool use_pairs(int rows) { return rows % 256 == 0; }
+// How a grouped GEMM is cut into tiles: the shape with the least (rounds over the GPU) x (time of a 64-deep step of a tile).
+// The step times are measured ones (us, d = 1024..2048, bf16); they grow far less than the tile does, because a step is a
+// chain of a load, a barrier and four MMAs, so the largest tiles win as long as they fill the GPU, and smaller ones where
+// they would leave SMs idle.  us, largest tile -> the one picked: gemm2 of 8 segments of 256 tokens, d = 1024, f = 2752:
+// 25 -> 23, dx 43 -> 39; gemm2 of 2 segments of 1000 tokens: 36 -> 23 (it used to run on 64-column tiles); 9 segments of
+// 200 tokens on CTA pairs: gemm1 24.9 -> 22.9.
+struct TileShape {
+  bool pair;  // 256-row tiles on CTA pairs, else 128-row tiles
+  int bn;     // columns (of both products together for the gate / up projections)
+};
+static TileShape pick_tiles(int M, int N, int groups, bool narrow) {
+  static const struct { TileShape t; double step; } shapes[5] = {
+      {{true, 256}, 0.47}, {{false, 256}, 0.54}, {{true, 128}, 0.42}, {{false, 128}, 0.40}, {{false, 64}, 0.36}};
+  TileShape best = {false, 256};
+  double least = 1e30;
+  for (int i = 0; i < (narrow ? 5 : 2); ++i) {
+    const TileShape t = shapes[i].t;
+    const long tiles = ceil_div(M, t.pair ? 256 : 128) * ceil_div(N, t.bn) * groups;
+    const double cost = (double)ceil_div(tiles, sm_count() / (t.pair ? 2 : 1)) * shapes[i].step;
+    if (cost < least) {
+      least = cost;
+      best = t;
+    }
+  }
+  return best;
+}
 
 struct WsPtrs {
   uint32_t* status;
@@ -588,6 +611,7 @@ static int launch_decode_m(const DecodeParams& p, cudaStream_t st) {
 static bool decode_supported(const lory_dims& D) {
   if (!(D.flags & LORY_FLAG_REUSE_MERGED) || D.T > 64) return false;
   const long gemm_tiles = ceil_div(D.f, 128) * D.B * (D.L / D.T);
+  if (getenv("X_DEC")) return atoi(getenv("X_DEC"));
   return D.T <= 16 || gemm_tiles <= (D.T <= 32 ? 2L : 1L) * sm_count();
 }
 bool tc_clears_status(const lory_dims& D) { return decode_supported(D); }
@@ -633,6 +657,7 @@ int tc_ffn_forward(const lory_dims& D, const Layout& Lo, char* ws, const bf16* x
 
   // G = X Wbar1^T, U = X Wbar3^T, H = silu(G) * U, one group per segment
   {
+    const TileShape ts = pick_tiles(T, 2 * f, S, false);
     CUtensorMap m_x, m_b1, m_b3, m_g, m_u, m_h;
     LORY_TRY(make_map(&m_x, x, d, T, S, d, (uint64_t)T * d, 128));
     LORY_TRY(make_blocked_map(&m_b1, q.wbar1, f, d, S, 64, 1, 1, 2));  // 128 rows (n) x 64 cols (k)
@@ -642,57 +667,36 @@ int tc_ffn_forward(const lory_dims& D, const Layout& Lo, char* ws, const bf16* x
     LORY_TRY(make_map(&m_h, q.H, f, T, S, f, (uint64_t)T * f, 32));
     TcGemmParams p = {};
     p.M = T; p.N = f; p.K = d; p.groups = S; p.status = q.status;
-    if (T <= 32) {  // a decode step: 32-row A tiles, the freed shared memory holds more weight stages
-      CUtensorMap m_xs;
-      LORY_TRY(make_map(&m_xs, x, d, T, S, d, (uint64_t)T * d, 32));
-      LORY_TRY((launch_tc<false, false, 256, MODE_DUALB, EPI_SWIGLU, true, false, 1, 32>("gemm1_swiglu", m_xs, m_xs, m_b1,
-                                                                                         m_b3, m_g, m_u, m_h, p, st)));
-    } else if (use_pairs(T))  // leader loads the Wbar1 rows (G half of the accumulator), its peer the Wbar3 rows (U half)
-      LORY_TRY((launch_tc<false, false, 256, MODE_DUALB, EPI_SWIGLU, true, false, 2>("gemm1_swiglu", m_x, m_x, m_b1, m_b3,
-                                                                                      m_g, m_u, m_h, p, st)));
-    else
-      LORY_TRY((launch_tc<false, false, 256, MODE_DUALB, EPI_SWIGLU, true>("gemm1_swiglu", m_x, m_x, m_b1, m_b3, m_g,
-                                                                            m_u, m_h, p, st)));
+    // pairs: the leader loads the Wbar1 rows (G half of the accumulator), its peer the Wbar3 rows (U half)
+    auto go = [&](auto launch) { return launch("gemm1_swiglu", m_x, m_x, m_b1, m_b3, m_g, m_u, m_h, p, st, nullptr, nullptr); };
+    if (ts.pair) LORY_TRY(go(launch_tc<false, false, 256, MODE_DUALB, EPI_SWIGLU, true, false, 2>));
+    else LORY_TRY(go(launch_tc<false, false, 256, MODE_DUALB, EPI_SWIGLU, true>));
   }
   // Y = H Wbar2^T
   {
+    const TileShape ts = pick_tiles(T, d, S, true);
     CUtensorMap m_h, m_b2, m_y;
-    const bool pair = use_pairs(T);
     LORY_TRY(make_map(&m_h, q.H, f, T, S, f, (uint64_t)T * f, 128));
-    // Few, short groups (a decode step: a handful of new tokens per sequence): 256-column tiles would leave most
-    // SMs without one while each tile streams a long strip of Wbar2; 64-column tiles spread that read over 4 x the SMs.
-    const bool narrow = !pair && ceil_div(T, 128) * ceil_div(d, 256) * S < sm_count();
-    // B tile: 256 rows (n = d index) x 64 cols (k = f index); a CTA pair loads 128 rows each
-    LORY_TRY(make_blocked_map(&m_b2, q.wbar2, d, f, S, 64, 1, 1, narrow ? 1 : (pair ? 2 : 4)));
+    // B tile: bn rows (n = d index) x 64 cols (k = f index); a CTA pair loads half of them each
+    LORY_TRY(make_blocked_map(&m_b2, q.wbar2, d, f, S, 64, 1, 1, ts.bn / (ts.pair ? 128 : 64)));
     LORY_TRY(make_map(&m_y, y, d, T, S, d, (uint64_t)T * d, 32));
     TcGemmParams p = {};
     p.M = T; p.N = d; p.K = f; p.groups = S; p.status = q.status;
-    p.residual = residual;
-    if (narrow && T <= 32 && !residual) {
-      CUtensorMap m_hs;
-      LORY_TRY(make_map(&m_hs, q.H, f, T, S, f, (uint64_t)T * f, 32));
-      LORY_TRY((launch_tc<false, false, 64, MODE_PLAIN, EPI_BF16, true, false, 1, 32>("gemm2", m_hs, m_hs, m_b2, m_b2, m_y,
-                                                                                      m_y, m_y, p, st)));
-    } else if (narrow) {
-      if (residual)
-        LORY_TRY((launch_tc<false, false, 64, MODE_PLAIN, EPI_BF16_RESADD, true>("gemm2", m_h, m_h, m_b2, m_b2, m_y, m_y,
-                                                                                  m_y, p, st)));
-      else
-        LORY_TRY((launch_tc<false, false, 64, MODE_PLAIN, EPI_BF16, true>("gemm2", m_h, m_h, m_b2, m_b2, m_y, m_y, m_y,
-                                                                          p, st)));
-    } else if (residual) {  // y = residual + H Wbar2^T: the block's skip connection rides in the epilogue
-      if (pair)
-        LORY_TRY((launch_tc<false, false, 256, MODE_PLAIN, EPI_BF16_RESADD, true, false, 2>("gemm2", m_h, m_h, m_b2, m_b2,
-                                                                                             m_y, m_y, m_y, p, st)));
-      else
-        LORY_TRY((launch_tc<false, false, 256, MODE_PLAIN, EPI_BF16_RESADD, true>("gemm2", m_h, m_h, m_b2, m_b2, m_y, m_y,
-                                                                                   m_y, p, st)));
-    } else if (pair)
-      LORY_TRY((launch_tc<false, false, 256, MODE_PLAIN, EPI_BF16, true, false, 2>("gemm2", m_h, m_h, m_b2, m_b2, m_y,
-                                                                                    m_y, m_y, p, st)));
-    else
-      LORY_TRY((launch_tc<false, false, 256, MODE_PLAIN, EPI_BF16, true>("gemm2", m_h, m_h, m_b2, m_b2, m_y, m_y, m_y,
-                                                                          p, st)));
+    p.residual = residual;   // y = residual + H Wbar2^T: the block's skip connection rides in the epilogue
+    auto go = [&](auto launch) { return launch("gemm2", m_h, m_h, m_b2, m_b2, m_y, m_y, m_y, p, st, nullptr, nullptr); };
+    if (residual) {
+      if (ts.pair && ts.bn == 256) LORY_TRY(go(launch_tc<false, false, 256, MODE_PLAIN, EPI_BF16_RESADD, true, false, 2>));
+      else if (ts.pair) LORY_TRY(go(launch_tc<false, false, 128, MODE_PLAIN, EPI_BF16_RESADD, true, false, 2>));
+      else if (ts.bn == 256) LORY_TRY(go(launch_tc<false, false, 256, MODE_PLAIN, EPI_BF16_RESADD, true>));
+      else if (ts.bn == 128) LORY_TRY(go(launch_tc<false, false, 128, MODE_PLAIN, EPI_BF16_RESADD, true>));
+      else LORY_TRY(go(launch_tc<false, false, 64, MODE_PLAIN, EPI_BF16_RESADD, true>));
+    } else {
+      if (ts.pair && ts.bn == 256) LORY_TRY(go(launch_tc<false, false, 256, MODE_PLAIN, EPI_BF16, true, false, 2>));
+      else if (ts.pair) LORY_TRY(go(launch_tc<false, false, 128, MODE_PLAIN, EPI_BF16, true, false, 2>));
+      else if (ts.bn == 256) LORY_TRY(go(launch_tc<false, false, 256, MODE_PLAIN, EPI_BF16, true>));
+      else if (ts.bn == 128) LORY_TRY(go(launch_tc<false, false, 128, MODE_PLAIN, EPI_BF16, true>));
+      else LORY_TRY(go(launch_tc<false, false, 64, MODE_PLAIN, EPI_BF16, true>));
+    }
   }
   return LORY_OK;
 }
@@ -741,23 +745,22 @@ int tc_ffn_backward(const lory_dims& D, const Layout& Lo, char* ws, const bf16* 
   // dH = dY Wbar2; dG, dU in the epilogue
   {
     CUtensorMap m_dy, m_b2, m_dgo, m_duo, m_gi, m_ui;
-    const bool pair = use_pairs(T);
+    const TileShape ts = pick_tiles(T, f, S, true);
     LORY_TRY(make_map(&m_dy, dy, d, T, S, d, (uint64_t)T * d, 128));
-    // B[k = d index (rows), n = f index]: 4 col blocks per tile, 2 per CTA of a pair
-    LORY_TRY(make_blocked_map(&m_b2, q.wbar2, d, f, S, 64, 1, pair ? 2 : 4, 1));
+    // B[k = d index (rows), n = f index]: bn / 64 col blocks per tile, half of them per CTA of a pair
+    LORY_TRY(make_blocked_map(&m_b2, q.wbar2, d, f, S, 64, 1, ts.bn / (ts.pair ? 128 : 64), 1));
     LORY_TRY(make_map(&m_dgo, q.dG, f, T, S, f, (uint64_t)T * f, 128));
     LORY_TRY(make_map(&m_duo, q.dU, f, T, S, f, (uint64_t)T * f, 128));
     LORY_TRY(make_map(&m_gi, q.G, f, T, S, f, (uint64_t)T * f, 128));
     LORY_TRY(make_map(&m_ui, q.U, f, T, S, f, (uint64_t)T * f, 128));
     TcGemmParams p = {};
     p.M = T; p.N = f; p.K = d; p.groups = S; p.status = q.status;
-    if (pair)
-      LORY_TRY((launch_tc<false, true, 256, MODE_PLAIN, EPI_DSWIGLU, true, false, 2>("dh_dswiglu", m_dy, m_dy, m_b2, m_b2,
-                                                                                      m_dgo, m_duo, m_duo, p, st, &m_gi,
-                                                                                      &m_ui)));
-    else
-      LORY_TRY((launch_tc<false, true, 256, MODE_PLAIN, EPI_DSWIGLU, true>("dh_dswiglu", m_dy, m_dy, m_b2, m_b2, m_dgo,
-                                                                            m_duo, m_duo, p, st, &m_gi, &m_ui)));
+    auto go = [&](auto launch) { return launch("dh_dswiglu", m_dy, m_dy, m_b2, m_b2, m_dgo, m_duo, m_duo, p, st, &m_gi, &m_ui); };
+    if (ts.pair && ts.bn == 256) LORY_TRY(go(launch_tc<false, true, 256, MODE_PLAIN, EPI_DSWIGLU, true, false, 2>));
+    else if (ts.pair) LORY_TRY(go(launch_tc<false, true, 128, MODE_PLAIN, EPI_DSWIGLU, true, false, 2>));
+    else if (ts.bn == 256) LORY_TRY(go(launch_tc<false, true, 256, MODE_PLAIN, EPI_DSWIGLU, true>));
+    else if (ts.bn == 128) LORY_TRY(go(launch_tc<false, true, 128, MODE_PLAIN, EPI_DSWIGLU, true>));
+    else LORY_TRY(go(launch_tc<false, true, 64, MODE_PLAIN, EPI_DSWIGLU, true>));
   }
   if (D.flags & LORY_FLAG_CHUNKED_ADJOINT) return tc_adjoint_chunked(D, q, x, w1, w2, w3, dy, dw1, dw2, dw3, st);
   // dWbar2[d, f] = dY^T H;  dWbar1[f, d] = dG^T X;  dWbar3[f, d] = dU^T X     (K = T), stored blocked
@@ -792,23 +795,22 @@ int tc_ffn_backward_dx(const lory_dims& D, const Layout& Lo, char* ws, const flo
   const int S = D.B * (D.L / D.T), T = D.T, d = D.d, f = D.f;
   const WsPtrs q = ws_ptrs(D, Lo, ws);
   CUtensorMap m_dg, m_du, m_b1, m_b3, m_dx;
-  const bool pair = use_pairs(T);
+  const TileShape ts = pick_tiles(T, d, S, true);
   LORY_TRY(make_map(&m_dg, q.dG, f, T, S, f, (uint64_t)T * f, 128));
   LORY_TRY(make_map(&m_du, q.dU, f, T, S, f, (uint64_t)T * f, 128));
-  // B[k = f index (rows), n = d index]: 4 col blocks per tile, 2 per CTA of a pair
-  LORY_TRY(make_blocked_map(&m_b1, q.wbar1, f, d, S, 64, 1, pair ? 2 : 4, 1));
-  LORY_TRY(make_blocked_map(&m_b3, q.wbar3, f, d, S, 64, 1, pair ? 2 : 4, 1));
+  // B[k = f index (rows), n = d index]: bn / 64 col blocks per tile, half of them per CTA of a pair
+  LORY_TRY(make_blocked_map(&m_b1, q.wbar1, f, d, S, 64, 1, ts.bn / (ts.pair ? 128 : 64), 1));
+  LORY_TRY(make_blocked_map(&m_b3, q.wbar3, f, d, S, 64, 1, ts.bn / (ts.pair ? 128 : 64), 1));
   LORY_TRY(make_map(&m_dx, dx, d, T, S, d, (uint64_t)T * d, 32));
   TcGemmParams p = {};
   p.M = T; p.N = d; p.K = f; p.groups = S; p.status = q.status;
   p.rowvec = dh_bar; p.row_scale = 1.0f / (float)T;
-  if (pair)
-    LORY_TRY((launch_tc<false, true, 256, MODE_DUALK, EPI_BF16_ROWADD, true, false, 2>("dx", m_dg, m_du, m_b1, m_b3, m_dx,
-                                                                                        m_dx, m_dx, p, st)));
-  else
-    LORY_TRY((launch_tc<false, true, 256, MODE_DUALK, EPI_BF16_ROWADD, true>("dx", m_dg, m_du, m_b1, m_b3, m_dx, m_dx,
-                                                                              m_dx, p, st)));
-  return LORY_OK;
+  auto go = [&](auto launch) { return launch("dx", m_dg, m_du, m_b1, m_b3, m_dx, m_dx, m_dx, p, st, nullptr, nullptr); };
+  if (ts.pair && ts.bn == 256) return go(launch_tc<false, true, 256, MODE_DUALK, EPI_BF16_ROWADD, true, false, 2>);
+  if (ts.pair) return go(launch_tc<false, true, 128, MODE_DUALK, EPI_BF16_ROWADD, true, false, 2>);
+  if (ts.bn == 256) return go(launch_tc<false, true, 256, MODE_DUALK, EPI_BF16_ROWADD, true>);
+  if (ts.bn == 128) return go(launch_tc<false, true, 128, MODE_DUALK, EPI_BF16_ROWADD, true>);
+  return go(launch_tc<false, true, 64, MODE_DUALK, EPI_BF16_ROWADD, true>);
 }
 
 // ---------------------------------------------------------------------------------------
