@@ -97,24 +97,26 @@ def _check(status):
 
 
 def _ptr(t):
+    # a plain integer: ctypes turns it into the void pointer the signature asks for, without an object per argument
     if t is None:
         return None
-    if hasattr(t, "data_ptr"):
+    try:
         if not t.is_contiguous():
             raise ValueError("tensors passed to the Lory library must be contiguous")
-        return ctypes.c_void_p(t.data_ptr())
-    return ctypes.c_void_p(int(t))
+        return t.data_ptr()
+    except AttributeError:
+        return int(t)
 
 
 def _nbytes(t):
-    return t.numel() * t.element_size()
+    return t.nbytes
 
 
 def _stream(stream):
     if stream is None:
         import torch
         stream = torch.cuda.current_stream()
-    return ctypes.c_void_p(getattr(stream, "cuda_stream", stream))
+    return getattr(stream, "cuda_stream", stream)
 
 
 def make_dims(B, L, T, d, f, E, dtype, flags=0):

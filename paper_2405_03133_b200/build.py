@@ -1,4 +1,5 @@
-"""Builds liblory.so (the C-ABI CUDA library) in-tree with nvcc for sm_100a.
+"""Builds liblory.so (the C-ABI CUDA library) in-tree with nvcc for sm_100a, and _torch_glue.so (the torch side of
+layer.py) with g++ against the installed torch.
 
     python -m paper_2405_03133_b200.build [--force] [-v] [--debug]
 """
@@ -12,6 +13,8 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "liblory.so")
+GLUE_SRC = os.path.join(HERE, "csrc_torch", "glue.cpp")
+GLUE = os.path.join(HERE, "_torch_glue.so")         # the torch side of layer.py (g++, no device code)
 LIB_DEBUG = os.path.join(HERE, "liblory_debug.so")   # the same sources with -DLORY_DEBUG (bounds checks in the kernels)
 SOURCES = ["lory_api.cu", "routing.cu", "simt.cu", "tc.cu", "noalloc.cu", "block.cu", "probe.cu"]
 NVCC_FLAGS = [
@@ -26,6 +29,31 @@ def _stale(lib) -> bool:
     t = os.path.getmtime(lib)
     deps = [os.path.join(CSRC, n) for n in os.listdir(CSRC)] + [os.path.join(ROOT, "include", "lory.h")]
     return any(os.path.getmtime(p) > t for p in deps)
+
+
+def build_glue(force: bool = False) -> str:
+    header = os.path.join(ROOT, "include", "lory.h")
+    if not force and os.path.exists(GLUE) and all(os.path.getmtime(p) <= os.path.getmtime(GLUE) for p in (GLUE_SRC, header)):
+        return GLUE
+    import sysconfig
+
+    import torch
+    from torch.utils import cpp_extension
+
+    cuda = os.environ.get("CUDA_HOME", "/usr/local/cuda")
+    inc = cpp_extension.include_paths() + [sysconfig.get_paths()["include"], os.path.join(cuda, "include"),
+                                           os.path.join(ROOT, "include")]
+    libdir = os.path.join(os.path.dirname(torch.__file__), "lib")
+    tmp = f"{GLUE}.{os.getpid()}"      # moved into place: another process may be importing the module
+    cmd = ([os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", "-DTORCH_EXTENSION_NAME=_torch_glue",
+            f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}"] + ["-I" + p for p in inc] + [GLUE_SRC] +
+           ["-L" + libdir, "-Wl,-rpath," + libdir, "-ltorch", "-ltorch_cpu", "-ltorch_cuda", "-ltorch_python", "-lc10",
+            "-lc10_cuda", "-ldl", "-o", tmp])
+    res = subprocess.run(cmd, capture_output=True, text=True)
+    if res.returncode != 0:
+        raise RuntimeError("g++ failed:\n" + res.stdout + res.stderr)
+    os.replace(tmp, GLUE)
+    return GLUE
 
 
 def build(force: bool = False, verbose: bool = False, debug: bool = False) -> str:
@@ -49,3 +77,4 @@ def build(force: bool = False, verbose: bool = False, debug: bool = False) -> st
 
 if __name__ == "__main__":
     print(build(force="--force" in sys.argv, verbose="-v" in sys.argv, debug="--debug" in sys.argv))
+    print(build_glue(force="--force" in sys.argv))

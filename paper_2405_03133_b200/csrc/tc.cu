@@ -602,7 +602,9 @@ static int launch_decode_m(const DecodeParams& p, cudaStream_t st) {
   const bool two = ceil_div(p.R, MODE == DECODE_16 ? 32 : 16) * p.S >= 6L * sm_count();
   if (p.n <= 8) return two ? launch_decode_t<MODE, 1, 2>(p, st) : launch_decode_t<MODE, 1, 1>(p, st);
   if (p.n <= 16) return two ? launch_decode_t<MODE, 2, 2>(p, st) : launch_decode_t<MODE, 2, 1>(p, st);
+  if (p.n <= 24) return launch_decode_t<MODE, 3, 2>(p, st);
   if (p.n <= 32) return launch_decode_t<MODE, 4, 2>(p, st);
+  if (p.n <= 48) return launch_decode_t<MODE, 6, 2>(p, st);
   return launch_decode_t<MODE, 8, 2>(p, st);
 }
 // Where the decode kernels run.  Past 16 tokens they fetch as many token as weight bytes, and the grouped GEMMs are the
@@ -611,7 +613,6 @@ static int launch_decode_m(const DecodeParams& p, cudaStream_t st) {
 static bool decode_supported(const lory_dims& D) {
   if (!(D.flags & LORY_FLAG_REUSE_MERGED) || D.T > 64) return false;
   const long gemm_tiles = ceil_div(D.f, 128) * D.B * (D.L / D.T);
-  if (getenv("X_DEC")) return atoi(getenv("X_DEC"));
   return D.T <= 16 || gemm_tiles <= (D.T <= 32 ? 2L : 1L) * sm_count();
 }
 bool tc_clears_status(const lory_dims& D) { return decode_supported(D); }
