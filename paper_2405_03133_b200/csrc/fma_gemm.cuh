@@ -94,6 +94,55 @@ __device__ __forceinline__ void fma2(float2& c, float a, const float2& b) {
   asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(cp) : "l"(ap), "l"(reinterpret_cast<const unsigned long long&>(b)));
 }
 
+// Finishes one row of a thread's outputs: v[j] are the four columns c0 + j * STEP of the CTA's tile (two products: the first
+// half of the j the gate, the second half the up values of the same columns).
+template <typename T, int MODE, int EPI, int JN, int STEP>
+__device__ __forceinline__ void fma_store_row(const FmaArgs& p, const FmaJob& J, float (&v)[JN][4], int g, int m, int n0, int c0,
+                                              bool vec) {
+  const size_t row = (size_t)g * J.c_g + (size_t)m * J.ldc;
+  if constexpr (EPI == FMA_SWIGLU) {
+#pragma unroll
+    for (int j = 0; j < JN / 2; ++j) {
+      const int n = n0 + c0 + j * STEP, left = J.N - n;
+      if (left <= 0) continue;
+      float h[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) h[i] = v[j][i] * sigmoidf_(v[j][i]) * v[j + JN / 2][i];
+      store4(static_cast<T*>(J.C0) + row + n, left, vec, v[j]);
+      store4(static_cast<T*>(J.C1) + row + n, left, vec, v[j + JN / 2]);
+      store4(static_cast<T*>(J.C2) + row + n, left, vec, h);
+    }
+  } else {
+#pragma unroll
+    for (int j = 0; j < JN; ++j) {
+      const int n = n0 + c0 + j * STEP, left = J.N - n;
+      if (left <= 0) continue;
+      if (EPI == FMA_DSWIGLU) {
+        float gg[4], uu[4], du[4];
+        load4(static_cast<const T*>(J.E0) + row + n, left, vec, gg);
+        load4(static_cast<const T*>(J.E1) + row + n, left, vec, uu);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const float s = sigmoidf_(gg[i]), dh = v[j][i];
+          v[j][i] = dh * uu[i] * s * (1.0f + gg[i] * (1.0f - s));
+          du[i] = dh * gg[i] * s;
+        }
+        store4(static_cast<T*>(J.C1) + row + n, left, vec, du);
+      } else if (EPI == FMA_ROWADD) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+          if (i < left) v[j][i] += p.rowvec[(size_t)g * J.N + n + i] * p.row_scale;
+      } else if (J.E0) {
+        float o[4];
+        load4(static_cast<const T*>(J.E0) + row + n, left, vec, o);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) v[j][i] += o[i];
+      }
+      store4(static_cast<T*>(J.C0) + row + n, left, vec, v[j]);
+    }
+  }
+}
+
 // A_K: A is stored [m][k] (else [k][m]); B_K: B is stored [n][k] (else [k][n]).  VEC: every row of A and B starts on a
 // 4-element boundary and has a multiple of 4 elements (one load and one predicate per four elements: 35 -> 48 TFLOP/s at
 // d = 768, f = 2064).
@@ -258,47 +307,154 @@ __global__ void __launch_bounds__(128 * KG, 3) fma_gemm_kernel(const __grid_cons
   for (int r = 0; r < MR; ++r) {
     const int m = m0 + (MR >= 4 ? (r >> 2) * 64 + ty * 4 + (r & 3) : ty * 2 + r);
     if (m >= J.M) continue;
-    const size_t row = (size_t)g * J.c_g + (size_t)m * J.ldc;
     float v[2][4] = {{acc[r][0].x, acc[r][0].y, acc[r][1].x, acc[r][1].y}, {acc[r][2].x, acc[r][2].y, acc[r][3].x, acc[r][3].y}};
-    if constexpr (EPI == FMA_SWIGLU) {
-      const int n = n0 + tx * 4, left = J.N - n;
-      if (left <= 0) continue;
-      float h[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) h[i] = v[0][i] * sigmoidf_(v[0][i]) * v[1][i];
-      store4(static_cast<T*>(J.C0) + row + n, left, vec, v[0]);
-      store4(static_cast<T*>(J.C1) + row + n, left, vec, v[1]);
-      store4(static_cast<T*>(J.C2) + row + n, left, vec, h);
+    fma_store_row<T, MODE, EPI, 2, 32>(p, J, v, g, m, n0, tx * 4, vec);
+  }
+}
+
+// -----------------------------------------------------------------------------------------------------------------
+// The same for fp32 operands and too few tiles to fill the GPU: 32 x 64 tiles whose contraction is shared by the eight warps
+// of a CTA, each with a cp.async ring of its own (transposing on the way where the contraction runs along the stored rows)
+// and no barrier until the end, where the warps' sums meet in shared memory and every warp finishes one row in eight.  A lane
+// computes 8 x 8 outputs, which needs a quarter of the shared-memory reads per FMA of the 2 x 8 above.  us, before -> after,
+// 8 segments of 128 tokens, d = 256, f = 688: gemm2 31 -> 27, dx 49 -> 33.
+// -----------------------------------------------------------------------------------------------------------------
+struct Fma32 {
+  static constexpr int KG = 8, BM = 32, BN = 64, BK = 16, STG = 3;
+  static constexpr int A_ROW = BM + 4, B_ROW = BN + 4, BLOCK = BK * (A_ROW + B_ROW);  // floats
+  static constexpr int SMEM = KG * STG * BLOCK * 4;
+};
+
+// A_K, B_K, VEC as above.
+template <bool A_K, bool B_K, int MODE, int EPI, bool VEC>
+__global__ void __launch_bounds__(32 * Fma32::KG, 1) fma32_kernel(const __grid_constant__ FmaArgs p) {
+  using F = Fma32;
+  constexpr int KG = F::KG, BK = F::BK, STG = F::STG, JN = 2;
+  constexpr int WA = VEC && !A_K ? 4 : 1, WB = VEC && !B_K ? 4 : 1;                // elements per copy
+  constexpr int NA = F::BM * BK / 32 / WA, NB = F::BN * BK / 32 / WB;              // copies per lane and block
+  constexpr int TILE_N = MODE == FMA_DUALB ? F::BN / 2 : F::BN;
+  extern __shared__ __align__(16) float s_tile[];   // [warp][stage][A: BK rows of A_ROW | B: BK rows of B_ROW]
+  const int kg = threadIdx.x >> 5, lane = threadIdx.x & 31, ty = lane >> 3, tx = lane & 7;
+  int tile = blockIdx.x, ji = 0;
+  while (ji + 1 < p.jobs && tile >= p.job[ji].tile_end) ++ji;
+  const FmaJob& J = p.job[ji];
+  tile -= ji ? p.job[ji - 1].tile_end : 0;
+  const int m0 = tile % J.m_tiles * F::BM, rest = tile / J.m_tiles, n0 = rest % J.n_tiles * TILE_N, g = rest / J.n_tiles;
+  const int nkb = (J.K + BK - 1) / BK, total = MODE == FMA_DUALK ? 2 * nkb : nkb;
+  const uint32_t ring = (uint32_t)__cvta_generic_to_shared(s_tile + kg * STG * F::BLOCK);
+
+  // Copy j of a block is element (k, x) of the tile, x along m or n; 1 or 4 elements along the contiguous dimension.  Where
+  // that is k, a warp takes eight k of four neighbouring x: 32-byte pieces of memory, 32 different banks.
+  auto at = [&](bool kc, int width, int w, int j, int& k, int& x) {
+    const int idx = lane + j * 32;
+    if (kc) {
+      x = (idx >> 3) % width;
+      k = (idx & 7) + 8 * ((idx >> 3) / width);
     } else {
+      x = idx % (width / w) * w;
+      k = idx / (width / w);
+    }
+  };
+  // Columns of the B tile: for two products, 32 of the first and the same 32 of the second.
+  auto b_col = [&](int x, bool& up) {
+    up = MODE == FMA_DUALB && x >= 32;
+    return n0 + (up ? x - 32 : x);
+  };
+  const float* const A0 = static_cast<const float*>(J.A0) + (size_t)g * J.a_g;
+  const float* const A1 = MODE == FMA_DUALK ? static_cast<const float*>(J.A1) + (size_t)g * J.a_g : A0;
+  const float* const B0 = static_cast<const float*>(J.B0) + (size_t)g * J.b_g;
+  const float* const B1 = MODE != FMA_PLAIN ? static_cast<const float*>(J.B1) + (size_t)g * J.b_g : B0;
+  auto copy = [&](uint32_t dst, const float* src, bool ok, int w) {   // outside the matrix: zeros
+    if (w == 4) asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(ok ? 16u : 0u) : "memory");
+    else asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst), "l"(src), "r"(ok ? 4u : 0u) : "memory");
+  };
+  auto issue = [&](int i, int st) {
+    if (i < total) {
+      const bool second = MODE == FMA_DUALK && i >= nkb;
+      const int k0 = (second ? i - nkb : i) * BK;
+      const float* const A = second ? A1 : A0;
+      const uint32_t sa = ring + st * F::BLOCK * 4, sb = sa + BK * F::A_ROW * 4;
 #pragma unroll
-      for (int half = 0; half < 2; ++half) {
-        const int n = n0 + half * 32 + tx * 4, left = J.N - n;
-        if (left <= 0) continue;
-        if (EPI == FMA_DSWIGLU) {
-          float gg[4], uu[4], du[4];
-          load4(static_cast<const T*>(J.E0) + row + n, left, vec, gg);
-          load4(static_cast<const T*>(J.E1) + row + n, left, vec, uu);
+      for (int j = 0; j < NA; ++j) {
+        int k, x;
+        at(A_K, F::BM, WA, j, k, x);
+        const int m = m0 + x, kk = k0 + k;
+        const bool ok = m < J.M && kk < J.K;
+        copy(sa + (k * F::A_ROW + x) * 4, ok ? A + (A_K ? m * J.lda + kk : kk * J.lda + m) : A0, ok, WA);
+      }
 #pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            const float s = sigmoidf_(gg[i]), dh = v[half][i];
-            v[half][i] = dh * uu[i] * s * (1.0f + gg[i] * (1.0f - s));
-            du[i] = dh * gg[i] * s;
-          }
-          store4(static_cast<T*>(J.C1) + row + n, left, vec, du);
-        } else if (EPI == FMA_ROWADD) {
-#pragma unroll
-          for (int i = 0; i < 4; ++i)
-            if (i < left) v[half][i] += p.rowvec[(size_t)g * J.N + n + i] * p.row_scale;
-        } else if (J.E0) {
-          float o[4];
-          load4(static_cast<const T*>(J.E0) + row + n, left, vec, o);
-#pragma unroll
-          for (int i = 0; i < 4; ++i) v[half][i] += o[i];
-        }
-        store4(static_cast<T*>(J.C0) + row + n, left, vec, v[half]);
+      for (int j = 0; j < NB; ++j) {
+        int k, x;
+        bool up;
+        at(B_K, F::BN, WB, j, k, x);
+        const int n = b_col(x, up), kk = k0 + k;
+        const bool ok = n < J.N && kk < J.K;
+        const float* const B = up || second ? B1 : B0;
+        copy(sb + (k * F::B_ROW + x) * 4, ok ? B + (B_K ? n * J.ldb + kk : kk * J.ldb + n) : B0, ok, WB);
       }
     }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+
+  float2 acc[8][2 * JN];   // rows ty * 4 + (r & 3) + (r >> 2) * 16, columns tx * 4 + j * 32
+#pragma unroll
+  for (int r = 0; r < 8; ++r)
+#pragma unroll
+    for (int j = 0; j < 2 * JN; ++j) acc[r][j] = make_float2(0.f, 0.f);
+#pragma unroll
+  for (int st = 0; st < STG - 1; ++st) issue(kg + st * KG, st);
+  int st = 0;
+  for (int i = kg; i < total; i += KG) {
+    asm volatile("cp.async.wait_group %0;" ::"n"(STG - 2) : "memory");
+    __syncwarp();   // the block is complete, and every lane is done with the stage that is filled next
+    issue(i + (STG - 1) * KG, st == 0 ? STG - 1 : st - 1);
+    const float* const sa = s_tile + (kg * STG + st) * F::BLOCK + ty * 4;
+    const float* const sb = s_tile + (kg * STG + st) * F::BLOCK + BK * F::A_ROW + tx * 4;
+    st = st + 1 == STG ? 0 : st + 1;
+#pragma unroll
+    for (int kk = 0; kk < BK; ++kk) {
+      float a[8];
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const float4 v = *reinterpret_cast<const float4*>(sa + kk * F::A_ROW + h * 16);
+        a[4 * h] = v.x; a[4 * h + 1] = v.y; a[4 * h + 2] = v.z; a[4 * h + 3] = v.w;
+      }
+      float2 b[2 * JN];
+#pragma unroll
+      for (int j = 0; j < JN; ++j) {
+        const float4 v = *reinterpret_cast<const float4*>(sb + kk * F::B_ROW + j * 32);
+        b[2 * j] = make_float2(v.x, v.y);
+        b[2 * j + 1] = make_float2(v.z, v.w);
+      }
+#pragma unroll
+      for (int r = 0; r < 8; ++r)
+#pragma unroll
+        for (int j = 0; j < 2 * JN; ++j) fma2(acc[r][j], a[r], b[j]);
+    }
   }
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
+  __syncthreads();   // the rings have been read
+#pragma unroll
+  for (int r = 0; r < 8; ++r)
+#pragma unroll
+    for (int j = 0; j < 2 * JN; ++j) {
+      s_tile[(kg * 64 + r * 8 + 2 * j) * 32 + lane] = acc[r][j].x;
+      s_tile[(kg * 64 + r * 8 + 2 * j + 1) * 32 + lane] = acc[r][j].y;
+    }
+  __syncthreads();
+  const int r = kg, m = m0 + ty * 4 + (r & 3) + (r >> 2) * 16;   // this warp's row of every lane's eight
+  if (m >= J.M) return;
+  float v[JN][4];
+#pragma unroll
+  for (int j = 0; j < JN; ++j)
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      float sum = 0.f;
+#pragma unroll
+      for (int q = 0; q < KG; ++q) sum += s_tile[(q * 64 + r * 8 + 4 * j + c) * 32 + lane];
+      v[j][c] = sum;
+    }
+  fma_store_row<float, MODE, EPI, JN, 32>(p, J, v, g, m, n0, tx * 4, J.vec != 0);
 }
 
 }  // namespace lory

@@ -97,49 +97,75 @@ static int sm_count_simt() {
   return n[dev];
 }
 
-// Tile choice.  128-row tiles have the best ratio of FMAs to shared-memory reads and need enough of them; below two per
-// SM 64-row tiles, below one per SM 32-row tiles (d = 256, f = 688, 8 segments of 128: dx 109, 60 and 44 us).  Two k-groups
-// per CTA where an SM gets fewer than three CTAs, and always with 32 rows, where a thread has too few FMAs between its
-// shared-memory reads to hide them (16-token segments, d = 301: 168 -> 136 us).
-template <typename T, bool A_K, bool B_K, int MODE, int EPI>
-static int fma_launch(FmaArgs a, int groups, cudaStream_t st) {
-  constexpr int TILE_N = MODE == FMA_DUALB ? 32 : 64;
-  const int sms = sm_count_simt();
-  auto count = [&](int bm) {
-    long t = 0;
-    for (int i = 0; i < a.jobs; ++i) t += ceil_div(a.job[i].M, bm) * ceil_div(a.job[i].N, TILE_N) * groups;
-    return t;
-  };
-  int mmax = 0;
-  for (int i = 0; i < a.jobs; ++i) mmax = a.job[i].M > mmax ? a.job[i].M : mmax;
-  const int bm = (mmax > 64 && count(128) >= 2L * sms) ? 128 : ((mmax > 32 && count(64) >= sms) ? 64 : 32);
-  const long tiles = count(bm);
-  if (tiles <= 0) return LORY_OK;
-  if (tiles > 0x7fffffffL) return LORY_ERR_SHAPE;
-  int acc = 0;
-  bool vec = true;
+// Fills in the tile counts of every job for tiles of bm x (columns of the outputs) tn; the number of tiles, or < 0.
+static long fma_tiles(FmaArgs& a, int groups, int bm, int tn) {
+  long acc = 0;
   for (int i = 0; i < a.jobs; ++i) {
     FmaJob& j = a.job[i];
     j.m_tiles = (int)ceil_div(j.M, bm);
-    j.n_tiles = (int)ceil_div(j.N, TILE_N);
-    acc += j.m_tiles * j.n_tiles * groups;
-    j.tile_end = acc;
+    j.n_tiles = (int)ceil_div(j.N, tn);
+    acc += (long)j.m_tiles * j.n_tiles * groups;
+    if (acc > 0x7fffffffL) return -1;
+    j.tile_end = (int)acc;
+  }
+  return acc;
+}
+// Whether inputs (returned) and outputs (FmaJob::vec) allow 4-element vectors.
+template <typename T, bool A_K, bool B_K>
+static bool fma_vectors(FmaArgs& a) {
+  bool vec = true;
+  for (int i = 0; i < a.jobs; ++i) {
+    FmaJob& j = a.job[i];
     const uintptr_t out = (uintptr_t)j.C0 | (uintptr_t)j.C1 | (uintptr_t)j.C2 | (uintptr_t)j.E0 | (uintptr_t)j.E1;
     j.vec = j.ldc % 4 == 0 && j.c_g % 4 == 0 && out % (4 * sizeof(T)) == 0;
     const uintptr_t in = (uintptr_t)j.A0 | (uintptr_t)j.A1 | (uintptr_t)j.B0 | (uintptr_t)j.B1;
     vec = vec && j.lda % 4 == 0 && j.ldb % 4 == 0 && j.a_g % 4 == 0 && j.b_g % 4 == 0 && in % (4 * sizeof(T)) == 0 &&
           (A_K ? j.K : j.M) % 4 == 0 && (B_K ? j.K : j.N) % 4 == 0;
   }
+  return vec;
+}
+template <bool A_K, bool B_K, int MODE, int EPI, bool VEC>
+static int launch_fma32(const FmaArgs& a, long tiles, cudaStream_t st) {
+  auto kern = fma32_kernel<A_K, B_K, MODE, EPI, VEC>;
+  static bool done[64];   // the attribute belongs to the (kernel, device) pair
+  int dev = 0;
+  LORY_CUDA_OK(cudaGetDevice(&dev));
+  if (dev < 0 || dev >= 64 || !done[dev]) {
+    LORY_CUDA_OK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, Fma32::SMEM));
+    if (dev >= 0 && dev < 64) done[dev] = true;
+  }
+  return launch_kernel(false, kern, dim3((unsigned)tiles), 32 * Fma32::KG, Fma32::SMEM, st, 1, a);
+}
+
+// Tile choice.  128-row tiles have the best ratio of FMAs to shared-memory reads and need enough of them; below two per
+// SM 64-row tiles, below one per SM 32-row tiles (d = 256, f = 688, 8 segments of 128: dx 109, 60 and 44 us).  Two k-groups
+// per CTA where an SM gets fewer than three CTAs, and always with 32 rows, where a thread has too few FMAs between its
+// shared-memory reads to hide them (16-token segments, d = 301: 168 -> 136 us).  fp32 with less than half a 64-row tile per
+// SM: the kernel that shares a 32-row tile's contraction between eight warps.
+template <typename T, bool A_K, bool B_K, int MODE, int EPI>
+static int fma_launch(FmaArgs a, int groups, cudaStream_t st) {
+  constexpr int TILE_N = MODE == FMA_DUALB ? 32 : 64;
+  const int sms = sm_count_simt();
+  int mmax = 0;
+  for (int i = 0; i < a.jobs; ++i) mmax = a.job[i].M > mmax ? a.job[i].M : mmax;
+  const long c128 = fma_tiles(a, groups, 128, TILE_N), c64 = fma_tiles(a, groups, 64, TILE_N);
+  const int bm = (mmax > 64 && c128 >= 2L * sms) ? 128 : ((mmax > 32 && c64 >= sms) ? 64 : 32);
+  const long tiles = fma_tiles(a, groups, bm, TILE_N);
+  if (tiles < 0) return LORY_ERR_SHAPE;
+  if (tiles == 0) return LORY_OK;
   const dim3 grid((unsigned)tiles);
   auto pick = [&](auto v) -> int {
     constexpr bool V = decltype(v)::value;
+    if constexpr (sizeof(T) == 4) {
+      if (bm == 32 && c64 * 2 < sms) return launch_fma32<A_K, B_K, MODE, EPI, V>(a, tiles, st);
+    }
     const bool two = bm == 32 || tiles < 3L * sms;
     if (bm == 128) return launch_kernel(false, fma_gemm_kernel<T, A_K, B_K, MODE, EPI, 128, 1, V>, grid, 128, 0, st, 1, a);
     if (bm == 64 && two) return launch_kernel(false, fma_gemm_kernel<T, A_K, B_K, MODE, EPI, 64, 2, V>, grid, 256, 0, st, 1, a);
     if (bm == 64) return launch_kernel(false, fma_gemm_kernel<T, A_K, B_K, MODE, EPI, 64, 1, V>, grid, 128, 0, st, 1, a);
     return launch_kernel(false, fma_gemm_kernel<T, A_K, B_K, MODE, EPI, 32, 2, V>, grid, 256, 0, st, 1, a);
   };
-  return vec ? pick(std::true_type()) : pick(std::false_type());
+  return fma_vectors<T, A_K, B_K>(a) ? pick(std::true_type()) : pick(std::false_type());
 }
 static FmaArgs one_job(const FmaJob& j) {
   FmaArgs a = {};
