@@ -163,7 +163,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__
   __shared__ uint32_t tmem_base_smem;
   __shared__ volatile uint32_t abort_flag;
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = ptx::warp_index(), lane = threadIdx.x & 31;
   const int num_tiles = p.m_tiles * p.n_tiles * p.groups;
 
   if (threadIdx.x == 0) {
@@ -203,7 +203,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__
 
   if (warp == 0) {
     // ------------------------------ TMA producer ------------------------------
-    if (lane == 0) {
+    if (ptx::elect_one()) {
       int s = 0;        // position in the stage ring and its phase, advanced by hand (no division per stage)
       uint32_t ph = 0;
       uint32_t issued = 0, last_parity = 0;
@@ -300,7 +300,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__
     }
   } else if (warp == 1) {
     // ------------------------------ MMA issuer ------------------------------
-    if (lane == 0 && rank == 0) {
+    if (rank == 0 && ptx::elect_one()) {
       constexpr uint32_t idesc = ptx::make_idesc_bf16(128 * CTAS, BN, A_MN, B_MN);
       // Shared-memory descriptors differ only in their 14-bit address field (16-byte units): the constant part is
       // built once, the stage ring advances by hand, and per MMA only an addition is left (measured neutral for

@@ -87,7 +87,7 @@ stage2_kernel(const __grid_constant__ Stage2Maps maps, const Stage2Params p) {
   __shared__ uint32_t tmem_base_smem;
   __shared__ volatile uint32_t abort_flag;
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = ptx::warp_index(), lane = threadIdx.x & 31;
   const int num_tiles = p.tile_end[2];
   const int STAGES = p.stages;
   const int NCB = p.ncb;   // 64-column blocks per tile (2; 3 on the fast path with 33..64 segments)
@@ -160,7 +160,7 @@ stage2_kernel(const __grid_constant__ Stage2Maps maps, const Stage2Params p) {
   };
 
   if (warp == 0) {
-    if (lane == 0) {
+    if (ptx::elect_one()) {
       // routing weights, once
       ptx::mbar_expect_tx(&w_bar, p.fast ? 65536u : (uint32_t)p.s_tiles * 32768u);
       if (p.fast) {
@@ -209,7 +209,7 @@ stage2_kernel(const __grid_constant__ Stage2Maps maps, const Stage2Params p) {
       }
     }
   } else if (warp == 1) {
-    if (lane == 0) {
+    if (ptx::elect_one()) {
       const uint32_t idesc1 = ptx::make_idesc_bf16(128, NCB * 64, true, true);
       if (!ptx::mbar_wait(&w_bar, 0, &abort_flag)) {
         atomicOr(p.status, STATUS_TIMEOUT_MMA);
@@ -269,7 +269,7 @@ stage2_kernel(const __grid_constant__ Stage2Maps maps, const Stage2Params p) {
     }
   } else if (warp == 6) {
     // the second product from a thread of its own (p.split)
-    if (lane == 0 && p.split) {
+    if (p.split && ptx::elect_one()) {
       const uint32_t stage16 = (uint32_t)p.stage_bytes >> 4;
       const uint32_t stage0_16 = ptx::smem_u32(s_stage) >> 4;
       const bool acc_ok = dbg::check(dbg::tmem_ok(tmem_d2, tmem_base, 512, (uint32_t)(p.s_tiles * p.Epad16)), p.status);

@@ -51,6 +51,16 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volati
   return false;
 }
 
+// The warp this thread is in, as a value the compiler knows to be the same for the whole warp, and one elected lane of a
+// converged warp.  TMA and MMA instructions take their operands from uniform registers: issued behind `if (lane == 0)`
+// they are compiled for the case that several lanes get there with different operands.
+__device__ __forceinline__ int warp_index() { return __shfl_sync(0xFFFFFFFFu, (int)threadIdx.x >> 5, 0); }
+__device__ __forceinline__ bool elect_one() {
+  uint32_t is;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xFFFFFFFF;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(is));
+  return is != 0;
+}
+
 // ---- TMA ------------------------------------------------------------------------------------
 __device__ __forceinline__ void prefetch_tmap(const void* tmap) {
   asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(tmap)) : "memory");

@@ -61,7 +61,7 @@ wgrad_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
   __shared__ uint32_t tmem_base_smem;
   __shared__ volatile uint32_t abort_flag;
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = ptx::warp_index(), lane = threadIdx.x & 31;
   const int nkb = (p.K + 63) / 64;                                  // <= KB_MAX (checked by the host)
   const int inner = RES_A ? p.n_tiles : p.m_tiles;                  // tiles of a strip
   const int num_strips = (RES_A ? p.m_tiles : p.n_tiles) * p.groups;
@@ -101,7 +101,7 @@ wgrad_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
 
   if (warp == 0) {
     // ------------------------------ TMA producer (one thread in each CTA) ------------------------------
-    if (lane == 0) {
+    if (ptx::elect_one()) {
       uint32_t it = 0, ri = 0;   // streamed pieces issued; strips started
       bool ok = true;
       // one piece: this CTA's 128 rows (A) or 128 columns (B) of a 64-token block = two boxes of 64
@@ -156,7 +156,7 @@ wgrad_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
     }
   } else if (warp == 1) {
     // ------------------------------ MMA issuer (leader CTA) ------------------------------
-    if (lane == 0 && rank == 0) {
+    if (rank == 0 && ptx::elect_one()) {
       constexpr uint32_t idesc = ptx::make_idesc_bf16(256, 256, true, true);
       const uint32_t res0 = ptx::smem_u32(s_res), ring0 = ptx::smem_u32(s_ring);
       uint32_t it = 0, ri = 0, tile_iter = 0;
