@@ -607,19 +607,54 @@ static int launch_decode_m(const DecodeParams& p, cudaStream_t st) {
   if (p.n <= 48) return launch_decode_t<MODE, 6, 2>(p, st);
   return launch_decode_t<MODE, 8, 2>(p, st);
 }
-// Where the decode kernels run.  Past 16 tokens they fetch as many token as weight bytes, and the grouped GEMMs are the
-// faster ones once these have the tiles to fill the GPU, twice over for up to 32 tokens (d = 1024, f = 2752, 24 tokens, 8
-// sequences: 47 -> 42 us, 16: 72 -> 80; 40 tokens, 4 sequences: 36 -> 30, 8: 47 -> 58).
-static bool decode_supported(const lory_dims& D) {
-  if (!(D.flags & LORY_FLAG_REUSE_MERGED) || D.T > 64) return false;
-  const long gemm_tiles = ceil_div(D.f, 128) * D.B * (D.L / D.T);
-  return D.T <= 16 || gemm_tiles <= (D.T <= 32 ? 2L : 1L) * sm_count();
+// 128 weight rows per tile; 64 for the down projection where whole ones would leave SMs idle (eight sequences of 40 tokens,
+// d = 1024: 36.1 -> 34.6 us a call).  Three blocks per stage where three such stages fit, else two: a stage's barriers cost
+// a fixed time (one block per stage: 39.2).
+template <bool GATE>
+static int launch_decode_mma(const lory_dims& D, const bf16* wa, const bf16* wb, const bf16* x, bf16* out, uint32_t* status, cudaStream_t st) {
+  DecodeMma p = {};
+  p.S = D.B * (D.L / D.T); p.n = D.T; p.R = GATE ? D.f : D.d; p.K = GATE ? D.d : D.f;
+  p.nb = (p.n + 15) / 16 * 16; p.out = out; p.status = status;
+  p.tr = GATE || ceil_div(p.R, 128) * p.S >= sm_count() ? 128 : 64;
+  const int kb_bytes = (p.tr + p.nb) * 128;
+  p.tail = GATE ? p.nb * p.tr / 2 * 4 : 0;
+  if (p.tail < 16384 - kb_bytes) p.tail = 16384 - kb_bytes;
+  const int room = kMaxSmem - 1024 - p.tail;   // 1024: alignment
+  p.kb = 9 * kb_bytes <= room ? 3 : 2;
+  const int stage = p.kb * kb_bytes;
+  p.stages = room / stage < 8 ? room / stage : 8;
+  CUtensorMap m_w, m_w3, m_x;
+  LORY_TRY(make_blocked_map(&m_w, wa, p.R, p.K, p.S, 64, 1, 1, !GATE && p.tr == 128 ? 2 : 1));
+  m_w3 = m_w;
+  if (GATE) LORY_TRY(make_blocked_map(&m_w3, wb, p.R, p.K, p.S, 64, 1, 1, 1));
+  LORY_TRY(make_map(&m_x, x, p.K, p.n, p.S, p.K, (uint64_t)p.n * p.K, p.nb));
+  static bool attr_set[kMaxDevices];
+  LORY_TRY(allow_dynamic_smem(decode_mma_kernel<GATE>, kMaxSmem, attr_set));
+  const long tiles = ceil_div(p.R, GATE ? 64 : p.tr) * p.S;
+  ProfScope ps(GATE ? "gemm1_swiglu" : "gemm2", st);
+  return launch_overlapped(decode_mma_kernel<GATE>, dim3((unsigned)(tiles < sm_count() ? tiles : sm_count())), 224,
+                           p.stages * stage + p.tail + 1024, st, 1, m_w, m_w3, m_x, p);
 }
-bool tc_clears_status(const lory_dims& D) { return decode_supported(D); }
+static bool decode_supported(const lory_dims& D) { return (D.flags & LORY_FLAG_REUSE_MERGED) && D.T <= 64; }
+// Past 16 tokens decode_kernel fetches as many token as weight bytes, and decode_mma_kernel takes over where its larger tiles
+// keep the SMs busy: past 32 tokens from half a tile per SM on, below from one and a half, and only with d > 512 (a tile of
+// fewer than three stages is all start and end).  us a call, decode_kernel or grouped GEMM -> decode_mma_kernel: 48 tokens, 4
+// sequences, d = 2048: 76 -> 55; 40, 8, d = 1024: 47 -> 35; 64, 1, d = 2048: 38 -> 33; 24, 8, d = 1024: 40 -> 33; on the other side
+// of the line 20, 1, d = 1024: 12 -> 19; 24, 2, d = 2048: 34 -> 39; 17, 32, d = 256: 16.5 -> 19.4.
+static bool decode_on_mma(const lory_dims& D) {
+  const long tiles = ceil_div(D.f, 64) * D.B * (D.L / D.T);
+  return D.T > 32 ? 2 * tiles >= sm_count() : D.T > 16 && D.d > 512 && 2 * tiles >= 3L * sm_count();
+}
+// (the debug build's bounds checks may report before a block of the same kernel has cleared the word)
+bool tc_clears_status(const lory_dims& D) { return decode_supported(D) && !(dbg::kOn && decode_on_mma(D)); }
 static int launch_decode(const lory_dims& D, const WsPtrs& q, const bf16* x, bf16* y, cudaStream_t st) {
   if ((uintptr_t)x & 15) {
     snprintf(call_state().cuda_error, sizeof(call_state().cuda_error), "x does not start on a 16-byte boundary");
     return LORY_ERR_CUDA;
+  }
+  if (decode_on_mma(D)) {
+    LORY_TRY(launch_decode_mma<true>(D, q.wbar1, q.wbar3, x, q.H, q.status, st));
+    return launch_decode_mma<false>(D, q.wbar2, nullptr, q.H, y, q.status, st);
   }
   DecodeParams p = {};
   p.wa = q.wbar1; p.wb = q.wbar3; p.x = x; p.out = q.H;

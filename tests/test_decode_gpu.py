@@ -17,7 +17,9 @@ pytestmark = pytest.mark.gpu
     (3, 72, 136, (1, 7, 16, 31, 32, 48)),      # rows and columns that end inside a 64 x 64 block
     (2, 584, 8, (1, 12, 40)),                  # more column blocks than warps, fewer rows than a tile
     (16, 640, 1024, (3, 16, 24)),              # several tiles per CTA; the down projection on 16-row tiles
-    (32, 896, 456, (8, 13, 20, 50)),           # two weight tiles at a time; the grouped GEMM from 33 tokens on
+    (32, 896, 456, (8, 13, 20, 50)),           # two weight tiles at a time
+    (32, 568, 456, (17, 32, 33, 64)),          # tcgen05: whole down-projection tiles, the last one half outside
+    (16, 72, 328, (32, 33, 48, 49)),           # tcgen05: two column blocks in a stage of three; half-filled gate tiles
 ])
 def test_decode_with_cached_merged_ffn(B, d, f, counts):
     wl = Workload("decode", B=B, L=64, T=64, d=d, f=f, E=3, dtype="bf16", w_r_std=2.0, seed=21)
