@@ -24,10 +24,9 @@
 // stream of ONE thread issuing both products (12 MMAs with their descriptors, 2 commits, 2 waits) was what a tile
 // waited for (E = 8, S = 128: 0.52 -> 0.45 ms; E = 16, S = 64, d = 2048: 1.83 -> 1.65 ms); each stage is handed back
 // once both threads' MMAs have read it (its barrier counts two arrivals).  A third issuer (the second product split
-// by column block into accumulators of their own) measured no faster.  Where the kernel waits for memory anyway
-// (more than 64 segments and more than 16 experts: E = 32, S = 128) the second issuer measured 5 % SLOWER on the
-// same GPU (0.57 -> 0.60 ms, 12 % more DRAM reads: tiles that share fetched lines drift apart), so there warp 1
-// issues both products (p.split = 0) and warp 6 idles.
+// by column block into accumulators of their own) measured no faster.  With many segments and experts the second
+// issuer pays once the clock has come down (E = 32, S = 128 in a steady loop: 577..625 -> 533..552 us; S = 256, d = 2048: 4.25 ->
+// 3.9 ms; on a cool GPU, where the kernel waits for memory alone, 0.51 -> 0.55 ms).
 #pragma once
 #include <cuda.h>
 
@@ -53,7 +52,6 @@ struct Stage2Params {
   int tile_end[3];  // exclusive prefix sums of (rows rounded up to 64) * ctiles
   int cb_stride;    // bytes between the two 64-column blocks of a dWbar tile in shared memory (= segments per box * 128)
   int dup;          // E <= 32: w_hi and w_lo are both the combined table [hi | lo | hi | hi | lo | lo] (32 columns each)
-  int split;        // the second product is issued by a warp of its own
   int fast;         // E <= 32 and S <= 64: hi and lo sums meet in the accumulator (see the kernel)
   int w_bytes;      // shared memory of the resident weight tiles
   int xch_bytes;    // one exchange buffer: 32 lanes x 256 B, or x 128 B with E <= 32
@@ -112,7 +110,7 @@ stage2_kernel(const __grid_constant__ Stage2Maps maps, const Stage2Params p) {
   if (threadIdx.x == 0) {
     for (int s = 0; s < 8; ++s) {
       ptx::mbar_init(&full_bar[s], 1);
-      ptx::mbar_init(&empty_bar[s], p.split ? 2 : 1);   // one arrival per MMA-issuing thread
+      ptx::mbar_init(&empty_bar[s], 2);   // one arrival per MMA-issuing thread
     }
     for (int a = 0; a < NACC; ++a) {
       ptx::mbar_init(&tmem_full_bar[a], 1);
@@ -223,11 +221,10 @@ stage2_kernel(const __grid_constant__ Stage2Maps maps, const Stage2Params p) {
       const uint32_t stage16 = (uint32_t)p.stage_bytes >> 4;
       const uint32_t stage0_16 = ptx::smem_u32(s_stage) >> 4, w16 = wbase >> 4;
       int s = 0;
-      uint32_t ph = 0, tcount = 0;
-      const bool d2_ok = dbg::check(dbg::tmem_ok(tmem_d2, tmem_base, 512, (uint32_t)(p.s_tiles * p.Epad16)), p.status);
+      uint32_t ph = 0;
       uint32_t acc = 0, acc_ph = 0;   // accumulator ring position and phase
       for (int tile = blockIdx.x; tile < num_tiles;
-           tile += gridDim.x, ++tcount, acc = (acc + 1 == NACC ? 0 : acc + 1), acc_ph ^= (acc == 0)) {
+           tile += gridDim.x, acc = (acc + 1 == NACC ? 0 : acc + 1), acc_ph ^= (acc == 0)) {
         if (!ptx::mbar_wait(&tmem_empty_bar[acc], acc_ph ^ 1, &abort_flag)) {
           atomicOr(p.status, STATUS_TIMEOUT_MMA);
           abort_flag = 1;
@@ -260,16 +257,14 @@ stage2_kernel(const __grid_constant__ Stage2Maps maps, const Stage2Params p) {
                              (st > 0 || kk > 0) ? 1u : 0u);
             }
           }
-          if (!p.split && d2_ok) issue_second(d16, st, tcount == 0);   // no second issuer: both products from here
           ptx::umma_commit(&empty_bar[s]);
         }
         ptx::umma_commit(&tmem_full_bar[acc]);
       }
-      if (!p.split) ptx::umma_commit(&d2_bar);
     }
   } else if (warp == 6) {
-    // the second product from a thread of its own (p.split)
-    if (p.split && ptx::elect_one()) {
+    // the second product from a thread of its own
+    if (ptx::elect_one()) {
       const uint32_t stage16 = (uint32_t)p.stage_bytes >> 4;
       const uint32_t stage0_16 = ptx::smem_u32(s_stage) >> 4;
       const bool acc_ok = dbg::check(dbg::tmem_ok(tmem_d2, tmem_base, 512, (uint32_t)(p.s_tiles * p.Epad16)), p.status);
