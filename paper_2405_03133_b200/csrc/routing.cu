@@ -12,6 +12,8 @@ namespace lory {
 // of it, a lane VEC consecutive columns (one 16-byte load per row).  Where there are too few segments to fill the GPU,
 // the blocks of a cluster (up to 8) share a segment's tokens and the first adds their sums through distributed shared
 // memory, in a fixed order (2 segments of 1000 tokens, d = 1024: 30 -> 4 us; with enough segments clusters only cost).
+// Another block's shared memory may be written only once that block is known to run: every block arrives at the cluster's
+// barrier first thing and waits on it right before its write, when all have long arrived.
 // ---------------------------------------------------------------------------------------
 template <typename T>
 struct Vec16;
@@ -46,6 +48,9 @@ __global__ void __launch_bounds__(256) pool_kernel(const T* __restrict__ x, floa
   const int col = (blockIdx.y * 32 + lane) * VEC;
   __shared__ float red[8][32 * VEC];
   __shared__ float xch[8][32 * VEC];   // the first block's: one row per block of the cluster
+  namespace cg = cooperative_groups;
+  cg::cluster_group cluster = cg::this_cluster();
+  if (parts > 1) cluster.barrier_arrive();
   pdl_launch();
   pdl_wait();
   if (status && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x < 64) status[threadIdx.x] = 0;
@@ -92,8 +97,7 @@ __global__ void __launch_bounds__(256) pool_kernel(const T* __restrict__ x, floa
     for (int w = 0; w < 8; ++w) sum += red[w][c];
   }
   if (parts > 1) {
-    namespace cg = cooperative_groups;
-    cg::cluster_group cluster = cg::this_cluster();
+    cluster.barrier_wait();   // the first block has started
     if (c < 32 * VEC) *cluster.map_shared_rank(&xch[part][c], 0) = sum;
     cluster.sync();
     if (part > 0) return;
