@@ -88,6 +88,22 @@ __device__ __forceinline__ void store4(T* p, int n, bool vec, const float (&v)[4
       if (i < n) p[i] = from_f32<T>(v[i]);
   }
 }
+// Addresses.  A group's activations [T, f] may have more than 2^31 elements, so element (row, col) lies at a 64-bit offset.
+// fma_row: with the pitch of a row in bytes, two instructions (row times elements, scaled afterwards, takes three).
+// fma_offset: from the start of a tile (at most 128 rows), whose own offset is 64-bit; 32 bits do there as long as a row
+// has fewer than 2^24 elements (WIDE otherwise).  Which one a kernel uses was measured: one load per element has no
+// registers left for the 64-bit rows (d = 1021, f = 2749: 6.45 ms a step against 5.90), the vector loads and the cp.async
+// rings would rather not form the tile's offset for every block (8 segments of 128 tokens, d = 256: 199 us against 183).
+template <typename T>
+__host__ __device__ __forceinline__ const T* fma_row(const T* p, int row, size_t pitch) {
+  return reinterpret_cast<const T*>(reinterpret_cast<const char*>(p) + (size_t)(unsigned)row * pitch);
+}
+template <bool WIDE>
+__host__ __device__ __forceinline__ long fma_offset(int row, int ld, int col) {
+  return WIDE ? (long)row * ld + col : (long)(row * ld + col);
+}
+__host__ __device__ __forceinline__ bool fma_wide(int ld) { return ld >= 1 << 24; }
+
 __device__ __forceinline__ void fma2(float2& c, float a, const float2& b) {
   unsigned long long ap, &cp = reinterpret_cast<unsigned long long&>(c);
   asm("mov.b64 %0, {%1, %1};" : "=l"(ap) : "f"(a));
@@ -145,8 +161,8 @@ __device__ __forceinline__ void fma_store_row(const FmaArgs& p, const FmaJob& J,
 
 // A_K: A is stored [m][k] (else [k][m]); B_K: B is stored [n][k] (else [k][n]).  VEC: every row of A and B starts on a
 // 4-element boundary and has a multiple of 4 elements (one load and one predicate per four elements: 35 -> 48 TFLOP/s at
-// d = 768, f = 2064).
-template <typename T, bool A_K, bool B_K, int MODE, int EPI, int BM, int KG, bool VEC>
+// d = 768, f = 2064).  WIDE: see fma_offset (without VEC only).
+template <typename T, bool A_K, bool B_K, int MODE, int EPI, int BM, int KG, bool VEC, bool WIDE = false>
 __global__ void __launch_bounds__(128 * KG, 3) fma_gemm_kernel(const __grid_constant__ FmaArgs p) {
   constexpr int BN = 64, BK = 16, MR = BM / 16, W = VEC ? 4 : 1;   // W: elements per load
   constexpr int NA = BM * BK / 128 / W, NB = BN * BK / 128 / W;    // loads per thread and block
@@ -181,6 +197,7 @@ __global__ void __launch_bounds__(128 * KG, 3) fma_gemm_kernel(const __grid_cons
   const T* const A1 = MODE == FMA_DUALK ? static_cast<const T*>(J.A1) + (size_t)g * J.a_g : A0;
   const T* const B0 = static_cast<const T*>(J.B0) + (size_t)g * J.b_g;
   const T* const B1 = MODE != FMA_PLAIN ? static_cast<const T*>(J.B1) + (size_t)g * J.b_g : B0;
+  const size_t pa = (size_t)J.lda * sizeof(T), pb = (size_t)J.ldb * sizeof(T);
   auto load_w = [&](const T* q, bool ok, float (&v)[W]) {
     if (VEC) {
       float t[4] = {0.f, 0.f, 0.f, 0.f};
@@ -194,21 +211,25 @@ __global__ void __launch_bounds__(128 * KG, 3) fma_gemm_kernel(const __grid_cons
   auto fetch = [&](int i) {
     const bool second = MODE == FMA_DUALK && i >= nkb;
     const int k0 = (second ? i - nkb : i) * BK;
-    const T* const A = second ? A1 : A0;
+    // VEC: rows and columns of the matrix; else of the tile, which starts at these offsets
+    const T* const A = (second ? A1 : A0) + (VEC ? 0 : fma_offset<true>(A_K ? m0 : k0, J.lda, A_K ? k0 : m0));
+    const long b0 = VEC ? 0 : fma_offset<true>(B_K ? n0 : k0, J.ldb, B_K ? k0 : n0);
+    auto elem = [&](const T* p, int r, int c, int ld, size_t pitch) { return VEC ? fma_row(p + c, r, pitch) : p + fma_offset<WIDE>(r, ld, c); };
 #pragma unroll
     for (int j = 0; j < NA; ++j) {
       int k, x;
       at(A_K, BM, j, k, x);
-      const int m = m0 + x, kk = k0 + k;
-      load_w(A + (A_K ? m * J.lda + kk : kk * J.lda + m), m < J.M && kk < J.K, ra[j]);
+      const int m = VEC ? m0 + x : x, kk = VEC ? k0 + k : k;
+      load_w(elem(A, A_K ? m : kk, A_K ? kk : m, J.lda, pa), m0 + x < J.M && k0 + k < J.K, ra[j]);
     }
 #pragma unroll
     for (int j = 0; j < NB; ++j) {
       int k, x;
       at(B_K, BN, j, k, x);
       const bool up = MODE == FMA_DUALB && x >= 32;
-      const int n = n0 + (up ? x - 32 : x), kk = k0 + k;
-      load_w((up || second ? B1 : B0) + (B_K ? n * J.ldb + kk : kk * J.ldb + n), n < J.N && kk < J.K, rb[j]);
+      const int xn = up ? x - 32 : x;
+      const int n = VEC ? n0 + xn : xn, kk = VEC ? k0 + k : k;
+      load_w(elem((up || second ? B1 : B0) + b0, B_K ? n : kk, B_K ? kk : n, J.ldb, pb), n0 + xn < J.N && k0 + k < J.K, rb[j]);
     }
   };
   auto put = [&](int buf) {
@@ -364,6 +385,7 @@ __global__ void __launch_bounds__(32 * Fma32::KG, 1) fma32_kernel(const __grid_c
   const float* const A1 = MODE == FMA_DUALK ? static_cast<const float*>(J.A1) + (size_t)g * J.a_g : A0;
   const float* const B0 = static_cast<const float*>(J.B0) + (size_t)g * J.b_g;
   const float* const B1 = MODE != FMA_PLAIN ? static_cast<const float*>(J.B1) + (size_t)g * J.b_g : B0;
+  const size_t pa = (size_t)J.lda * sizeof(float), pb = (size_t)J.ldb * sizeof(float);
   auto copy = [&](uint32_t dst, const float* src, bool ok, int w) {   // outside the matrix: zeros
     if (w == 4) asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(ok ? 16u : 0u) : "memory");
     else asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst), "l"(src), "r"(ok ? 4u : 0u) : "memory");
@@ -380,7 +402,7 @@ __global__ void __launch_bounds__(32 * Fma32::KG, 1) fma32_kernel(const __grid_c
         at(A_K, F::BM, WA, j, k, x);
         const int m = m0 + x, kk = k0 + k;
         const bool ok = m < J.M && kk < J.K;
-        copy(sa + (k * F::A_ROW + x) * 4, ok ? A + (A_K ? m * J.lda + kk : kk * J.lda + m) : A0, ok, WA);
+        copy(sa + (k * F::A_ROW + x) * 4, ok ? fma_row(A + (A_K ? kk : m), A_K ? m : kk, pa) : A0, ok, WA);
       }
 #pragma unroll
       for (int j = 0; j < NB; ++j) {
@@ -390,7 +412,7 @@ __global__ void __launch_bounds__(32 * Fma32::KG, 1) fma32_kernel(const __grid_c
         const int n = b_col(x, up), kk = k0 + k;
         const bool ok = n < J.N && kk < J.K;
         const float* const B = up || second ? B1 : B0;
-        copy(sb + (k * F::B_ROW + x) * 4, ok ? B + (B_K ? n * J.ldb + kk : kk * J.ldb + n) : B0, ok, WB);
+        copy(sb + (k * F::B_ROW + x) * 4, ok ? fma_row(B + (B_K ? kk : n), B_K ? n : kk, pb) : B0, ok, WB);
       }
     }
     asm volatile("cp.async.commit_group;" ::: "memory");

@@ -147,9 +147,14 @@ static int fma_launch(FmaArgs a, int groups, cudaStream_t st) {
   constexpr int TILE_N = MODE == FMA_DUALB ? 32 : 64;
   const int sms = sm_count_simt();
   int mmax = 0;
-  for (int i = 0; i < a.jobs; ++i) mmax = a.job[i].M > mmax ? a.job[i].M : mmax;
+  const bool vec = fma_vectors<T, A_K, B_K>(a);
+  bool wide = false;   // rows too long for 32-bit offsets inside a tile: one general shape
+  for (int i = 0; i < a.jobs; ++i) {
+    mmax = a.job[i].M > mmax ? a.job[i].M : mmax;
+    wide = wide || (!vec && (fma_wide(a.job[i].lda) || fma_wide(a.job[i].ldb)));
+  }
   const long c128 = fma_tiles(a, groups, 128, TILE_N), c64 = fma_tiles(a, groups, 64, TILE_N);
-  const int bm = (mmax > 64 && c128 >= 2L * sms) ? 128 : ((mmax > 32 && c64 >= sms) ? 64 : 32);
+  const int bm = wide ? 32 : (mmax > 64 && c128 >= 2L * sms) ? 128 : ((mmax > 32 && c64 >= sms) ? 64 : 32);
   const long tiles = fma_tiles(a, groups, bm, TILE_N);
   if (tiles < 0) return LORY_ERR_SHAPE;
   if (tiles == 0) return LORY_OK;
@@ -159,13 +164,16 @@ static int fma_launch(FmaArgs a, int groups, cudaStream_t st) {
     if constexpr (sizeof(T) == 4) {
       if (bm == 32 && c64 * 2 < sms) return launch_fma32<A_K, B_K, MODE, EPI, V>(a, tiles, st);
     }
+    if constexpr (!V) {
+      if (wide) return launch_kernel(false, fma_gemm_kernel<T, A_K, B_K, MODE, EPI, 32, 2, V, true>, grid, 256, 0, st, 1, a);
+    }
     const bool two = bm == 32 || tiles < 3L * sms;
     if (bm == 128) return launch_kernel(false, fma_gemm_kernel<T, A_K, B_K, MODE, EPI, 128, 1, V>, grid, 128, 0, st, 1, a);
     if (bm == 64 && two) return launch_kernel(false, fma_gemm_kernel<T, A_K, B_K, MODE, EPI, 64, 2, V>, grid, 256, 0, st, 1, a);
     if (bm == 64) return launch_kernel(false, fma_gemm_kernel<T, A_K, B_K, MODE, EPI, 64, 1, V>, grid, 128, 0, st, 1, a);
     return launch_kernel(false, fma_gemm_kernel<T, A_K, B_K, MODE, EPI, 32, 2, V>, grid, 256, 0, st, 1, a);
   };
-  return fma_vectors<T, A_K, B_K>(a) ? pick(std::true_type()) : pick(std::false_type());
+  return vec ? pick(std::true_type()) : pick(std::false_type());
 }
 static FmaArgs one_job(const FmaJob& j) {
   FmaArgs a = {};
