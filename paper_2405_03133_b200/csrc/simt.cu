@@ -331,6 +331,7 @@ __global__ void __launch_bounds__(256) fma_adjoint_kernel(const __grid_constant_
           *q = from_f32<T>(p.accumulate ? acc[e] + to_f32(*q) : acc[e]);
         }
     }
+    const unsigned mask = __ballot_sync(0xffffffffu, sg * 4 < ns);   // the lanes that go in (eg is the warp's)
     if (sg * 4 < ns && eg * EB < p.E) {
       float dot[4][EB];
 #pragma unroll
@@ -350,8 +351,6 @@ __global__ void __launch_bounds__(256) fma_adjoint_kernel(const __grid_constant_
             dot[i][e] = fmaf(d4[i].x, w4.x, fmaf(d4[i].y, w4.y, fmaf(d4[i].z, w4.z, fmaf(d4[i].w, w4.w, dot[i][e]))));
         }
       }
-      // the four lanes of a segment group are in here together
-      const unsigned mask = __activemask();
 #pragma unroll
       for (int i = 0; i < 4; ++i)
 #pragma unroll

@@ -21,3 +21,9 @@ def test_distributed_shared_memory_is_touched_after_a_cluster_barrier(name):
         if "map_shared_rank" in body:
             before = body[:body.index("map_shared_rank")]
             assert re.search(r"\.sync\(\)|barrier_wait\(", before), body[:200]
+
+
+@pytest.mark.parametrize("name", sorted(n for n in os.listdir(CSRC) if n.endswith((".cu", ".cuh"))))
+def test_no_mask_is_taken_from_whoever_happens_to_be_there(name):
+    """__activemask() says which lanes are converged, not which will take part: no argument for a warp-wide exchange."""
+    assert not any("__activemask" in body for body in kernels(name))
