@@ -99,6 +99,29 @@ Forward run_forward(const lory_dims& d, const Tensor& x, const Tensor& gamma, co
   return r;
 }
 
+struct Grads {
+  Tensor dx, dgamma, dw_r, dW1, dW2, dW3;
+};
+Grads run_backward(const lory_dims& d, const Tensor& x, const Tensor& gamma, const Tensor& w_r, const Tensor& W1,
+                   const Tensor& W2, const Tensor& W3, const Tensor& ws, const Tensor& dy) {
+  Grads g;
+  g.dx = at::empty_like(x);
+  g.dw_r = at::empty_like(w_r);
+  g.dW1 = at::empty_like(W1);
+  g.dW2 = at::empty_like(W2);
+  g.dW3 = at::empty_like(W3);
+  const size_t n = (size_t)ws.numel();
+  if (gamma.defined()) {
+    g.dgamma = at::empty_like(gamma);
+    ok(api.block_backward(&d, ptr(x), ptr(gamma), ptr(w_r), ptr(W1), ptr(W2), ptr(W3), ptr(dy), ptr(g.dx), ptr(g.dgamma),
+                          ptr(g.dw_r), ptr(g.dW1), ptr(g.dW2), ptr(g.dW3), nullptr, ptr(ws), n, stream_of(x)));
+  } else {
+    ok(api.backward(&d, ptr(x), ptr(w_r), ptr(W1), ptr(W2), ptr(W3), ptr(dy), ptr(g.dx), ptr(g.dw_r), ptr(g.dW1), ptr(g.dW2),
+                    ptr(g.dW3), nullptr, ptr(ws), n, stream_of(x)));
+  }
+  return g;
+}
+
 struct LoryFunction : torch::autograd::Function<LoryFunction> {
   static variable_list forward(AutogradContext* ctx, const Variable& x_in, const c10::optional<Tensor>& gamma_in,
                                const Variable& w_r, const Variable& W1, const Variable& W2, const Variable& W3, int64_t T,
@@ -122,20 +145,9 @@ struct LoryFunction : torch::autograd::Function<LoryFunction> {
     TORCH_CHECK(ctx->saved_data.count("ws"), "the layer's saved activations have been used by an earlier backward");
     const Tensor ws = ctx->saved_data["ws"].toTensor();
     const lory_dims d = dims_of(x, W1, ctx->saved_data["T"].toInt(), ctx->saved_data["flags"].toInt());
-    const Tensor dy = grads[0].contiguous();
-    Tensor dx = at::empty_like(x), dgamma, dw_r = at::empty_like(w_r), dW1 = at::empty_like(W1), dW2 = at::empty_like(W2),
-           dW3 = at::empty_like(W3);
-    const size_t n = (size_t)ws.numel();
-    if (gamma.defined()) {
-      dgamma = at::empty_like(gamma);
-      ok(api.block_backward(&d, ptr(x), ptr(gamma), ptr(w_r), ptr(W1), ptr(W2), ptr(W3), ptr(dy), ptr(dx), ptr(dgamma),
-                            ptr(dw_r), ptr(dW1), ptr(dW2), ptr(dW3), nullptr, ptr(ws), n, stream_of(x)));
-    } else {
-      ok(api.backward(&d, ptr(x), ptr(w_r), ptr(W1), ptr(W2), ptr(W3), ptr(dy), ptr(dx), ptr(dw_r), ptr(dW1), ptr(dW2),
-                      ptr(dW3), nullptr, ptr(ws), n, stream_of(x)));
-    }
+    const Grads g = run_backward(d, x, gamma, w_r, W1, W2, W3, ws, grads[0].contiguous());
     ctx->saved_data.erase("ws");
-    return {dx, dgamma, dw_r, dW1, dW2, dW3, Tensor(), Tensor(), Tensor()};
+    return {g.dx, g.dgamma, g.dw_r, g.dW1, g.dW2, g.dW3, Tensor(), Tensor(), Tensor()};
   }
 };
 
@@ -153,6 +165,25 @@ std::tuple<Tensor, Tensor> moe(const Tensor& x, const c10::optional<Tensor>& gam
   }
   auto out = LoryFunction::apply(x, gamma, w_r, W1, W2, W3, T, eps, flags);
   return {out[0], out[1]};
+}
+
+// The two halves without a node of their own, for a node in Python (see layer.py): x and dy contiguous; the workspace is the
+// backward's if `keep`.
+std::tuple<Tensor, Tensor, Tensor> forward(const Tensor& x, const c10::optional<Tensor>& gamma, const Tensor& w_r,
+                                           const Tensor& W1, const Tensor& W2, const Tensor& W3, int64_t T, double eps,
+                                           int64_t flags, bool keep) {
+  py::gil_scoped_release no_gil;
+  c10::cuda::CUDAGuard guard(x.device());
+  Forward r = run_forward(dims_of(x, W1, T, flags), x, gamma.value_or(Tensor()), w_r, W1, W2, W3, eps, keep);
+  return {r.y, r.route_w, r.ws};
+}
+std::vector<c10::optional<Tensor>> backward(const Tensor& x, const c10::optional<Tensor>& gamma, const Tensor& w_r,
+                                            const Tensor& W1, const Tensor& W2, const Tensor& W3, const Tensor& ws,
+                                            const Tensor& dy, int64_t T, int64_t flags) {
+  py::gil_scoped_release no_gil;
+  c10::cuda::CUDAGuard guard(x.device());
+  const Grads g = run_backward(dims_of(x, W1, T, flags), x, gamma.value_or(Tensor()), w_r, W1, W2, W3, ws, dy);
+  return {g.dx, gamma.has_value() ? c10::optional<Tensor>(g.dgamma) : c10::nullopt, g.dw_r, g.dW1, g.dW2, g.dW3};
 }
 
 // Prompt-only routing: one segment per sequence; the workspace keeps the merged weights.
@@ -187,6 +218,8 @@ Tensor decode(const Tensor& x_in, const Tensor& W1, const Tensor& W2, const Tens
 PYBIND11_MODULE(_torch_glue, m) {
   m.def("bind", &bind);
   m.def("moe", &moe);
+  m.def("forward", &forward);
+  m.def("backward", &backward);
   m.def("prefill", &prefill);
   m.def("decode", &decode);
 }

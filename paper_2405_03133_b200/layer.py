@@ -34,6 +34,32 @@ def _load_glue():
 _glue = _load_glue()
 
 
+class _TracedFunction(torch.autograd.Function):
+    """The same node in Python, for torch.jit.trace: it records a Python function as one operation, while of the C++ one it
+    would record the allocation of the outputs and not what fills them."""
+
+    @staticmethod
+    def forward(ctx, x, gamma, w_r, W1, W2, W3, T, eps, flags):
+        x = x.contiguous()
+        keep = any(ctx.needs_input_grad)
+        y, route_w, ws = _glue.forward(x, gamma, w_r, W1, W2, W3, T, eps, flags, keep)
+        if keep:
+            ctx.save_for_backward(x, gamma, w_r, W1, W2, W3)
+            ctx.ws, ctx.T, ctx.flags = ws, T, flags
+        ctx.mark_non_differentiable(route_w)
+        return y, route_w
+
+    @staticmethod
+    def backward(ctx, dy, _d_route_w):
+        grads = _glue.backward(*ctx.saved_tensors, ctx.ws, dy.contiguous(), ctx.T, ctx.flags)
+        ctx.ws = None
+        return *grads, None, None, None
+
+
+def _moe(*args):
+    return _TracedFunction.apply(*args) if torch.jit.is_tracing() else _glue.moe(*args)
+
+
 class LoryMoE(torch.nn.Module):
     """Lory mixture-of-experts FFN layer (causal segment routing + expert merging, Sections 3 and 3.1).
 
@@ -60,7 +86,7 @@ class LoryMoE(torch.nn.Module):
     def forward(self, x: torch.Tensor) -> torch.Tensor:
         if not x.is_cuda:
             raise RuntimeError("LoryMoE runs on a CUDA device only (there is no CPU path)")
-        y, self.last_route_w = _glue.moe(x, None, self.w_r, self.W1, self.W2, self.W3, self.T, 0.0, self.flags)
+        y, self.last_route_w = _moe(x, None, self.w_r, self.W1, self.W2, self.W3, self.T, 0.0, self.flags)
         return y
 
 
@@ -77,7 +103,7 @@ class LoryBlock(LoryMoE):
     def forward(self, x: torch.Tensor) -> torch.Tensor:
         if not x.is_cuda:
             raise RuntimeError("LoryBlock runs on a CUDA device only (there is no CPU path)")
-        y, self.last_route_w = _glue.moe(x, self.gamma, self.w_r, self.W1, self.W2, self.W3, self.T, self.eps, self.flags)
+        y, self.last_route_w = _moe(x, self.gamma, self.w_r, self.W1, self.W2, self.W3, self.T, self.eps, self.flags)
         return y
 
 
