@@ -154,6 +154,10 @@ struct LoryFunction : torch::autograd::Function<LoryFunction> {
 std::tuple<Tensor, Tensor> moe(const Tensor& x, const c10::optional<Tensor>& gamma, const Tensor& w_r, const Tensor& W1,
                                const Tensor& W2, const Tensor& W3, int64_t T, double eps, int64_t flags) {
   py::gil_scoped_release no_gil;
+  // with or without gradients: a tangent must not get lost
+  bool dual = gamma.has_value() && gamma->_fw_grad(0).defined();
+  for (const Tensor* t : {&x, &w_r, &W1, &W2, &W3}) dual = dual || t->_fw_grad(0).defined();
+  TORCH_CHECK_NOT_IMPLEMENTED(!dual, "the Lory layer has no forward-mode derivative");
   const bool grad = at::GradMode::is_enabled() &&
                     (x.requires_grad() || w_r.requires_grad() || W1.requires_grad() || W2.requires_grad() ||
                      W3.requires_grad() || (gamma.has_value() && gamma->requires_grad()));

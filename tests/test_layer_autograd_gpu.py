@@ -36,6 +36,16 @@ def test_traced_module_computes_for_other_inputs(cls, grad):
         assert all(torch.equal(a, b) for a, b in zip(ga, gb))
 
 
+@pytest.mark.parametrize("grad,frozen", [(True, False), (True, True), (False, False)])
+def test_forward_mode_is_refused(grad, frozen):
+    m = layer(frozen=frozen)
+    with torch.autograd.forward_ad.dual_level(), torch.set_grad_enabled(grad):
+        x = torch.autograd.forward_ad.make_dual(tokens(2), tokens(3))
+        with pytest.raises(NotImplementedError):
+            m(x)
+        m(tokens(4))                        # no tangent, no objection
+
+
 @pytest.mark.parametrize("frozen", [False, True])
 def test_function_transforms_are_refused(frozen):
     m = layer(frozen=frozen)
