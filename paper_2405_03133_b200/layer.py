@@ -12,26 +12,40 @@ smaller forward-only one and is dropped at once.
 """
 from __future__ import annotations
 
+import importlib
+import threading
+
 import torch
 
 from . import binding as _lory
 
 
-def _load_glue():
-    """The C++ side of this file (autograd nodes, allocations, argument marshalling), built on first use if need be."""
-    import importlib
-    try:
-        glue = importlib.import_module("._torch_glue", __package__)
-    except ImportError:
-        from . import build
-        build.build_glue(force=True)
-        glue = importlib.import_module("._torch_glue", __package__)
-    _lory.load()
-    glue.bind(_lory.LIB_PATH, _lory._check)
-    return glue
+_module = None
+_lock = threading.Lock()
 
 
-_glue = _load_glue()
+def _glue():
+    """The C++ side of this file (autograd nodes, allocations, argument marshalling): loaded by the first call that needs it,
+    and built before that if need be."""
+    if _module is None:
+        _load()
+    return _module
+
+
+def _load():
+    global _module
+    with _lock:
+        if _module is not None:
+            return
+        _lory.load()
+        try:
+            glue = importlib.import_module("._torch_glue", __package__)
+        except ImportError:
+            from . import build
+            build.build_glue(force=True)
+            glue = importlib.import_module("._torch_glue", __package__)
+        glue.bind(_lory.LIB_PATH, _lory._check)
+        _module = glue
 
 
 class _TracedFunction(torch.autograd.Function):
@@ -42,7 +56,7 @@ class _TracedFunction(torch.autograd.Function):
     def forward(ctx, x, gamma, w_r, W1, W2, W3, T, eps, flags):
         x = x.contiguous()
         keep = any(ctx.needs_input_grad)
-        y, route_w, ws = _glue.forward(x, gamma, w_r, W1, W2, W3, T, eps, flags, keep)
+        y, route_w, ws = _glue().forward(x, gamma, w_r, W1, W2, W3, T, eps, flags, keep)
         if keep:
             ctx.save_for_backward(x, gamma, w_r, W1, W2, W3)
             ctx.ws, ctx.T, ctx.flags = ws, T, flags
@@ -51,13 +65,13 @@ class _TracedFunction(torch.autograd.Function):
 
     @staticmethod
     def backward(ctx, dy, _d_route_w):
-        grads = _glue.backward(*ctx.saved_tensors, ctx.ws, dy.contiguous(), ctx.T, ctx.flags)
+        grads = _glue().backward(*ctx.saved_tensors, ctx.ws, dy.contiguous(), ctx.T, ctx.flags)
         ctx.ws = None
         return *grads, None, None, None
 
 
 def _moe(*args):
-    return _TracedFunction.apply(*args) if torch.jit.is_tracing() else _glue.moe(*args)
+    return _TracedFunction.apply(*args) if torch.jit.is_tracing() else _glue().moe(*args)
 
 
 class LoryMoE(torch.nn.Module):
@@ -121,7 +135,7 @@ class LoryPromptRoutedFFN:
         m = self.layer
         # on the stream torch is issuing this tensor's work on, so that the call is ordered with its producers and
         # consumers (and with later decode() calls, which share the cached workspace)
-        y, self.route_w, self.ws = _glue.prefill(x_prompt, m.w_r, m.W1, m.W2, m.W3, m.flags)
+        y, self.route_w, self.ws = _glue().prefill(x_prompt, m.w_r, m.W1, m.W2, m.W3, m.flags)
         self.batch = x_prompt.shape[0]
         return y
 
@@ -131,4 +145,4 @@ class LoryPromptRoutedFFN:
         if x_new.shape[0] != self.batch:
             raise ValueError("decode() needs the batch of the prefill() whose merged FFNs are cached")
         m = self.layer
-        return _glue.decode(x_new, m.W1, m.W2, m.W3, self.ws, m.flags)
+        return _glue().decode(x_new, m.W1, m.W2, m.W3, self.ws, m.flags)
