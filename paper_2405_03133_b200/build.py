@@ -5,6 +5,7 @@ layer.py) with g++ against the installed torch.
 """
 from __future__ import annotations
 
+import hashlib
 import os
 import subprocess
 import sys
@@ -31,9 +32,26 @@ def _stale(lib) -> bool:
     return any(os.path.getmtime(p) > t for p in deps)
 
 
+def glue_tag() -> str:
+    """What the glue was built from: its sources, the C ABI it calls and the torch it is linked to."""
+    import torch
+    h = hashlib.sha256(torch.__version__.encode())
+    for path in (GLUE_SRC, os.path.join(ROOT, "include", "lory.h")):
+        with open(path, "rb") as f:
+            h.update(f.read())
+    return "lory-glue-" + h.hexdigest()
+
+
+def glue_is_current() -> bool:
+    """Whether _torch_glue.so carries the tag of the sources (asked of the file: a module once loaded cannot be replaced)."""
+    if not os.path.exists(GLUE) or not os.path.exists(GLUE_SRC):
+        return os.path.exists(GLUE)     # without sources there is nothing to compare with
+    with open(GLUE, "rb") as f:
+        return glue_tag().encode() in f.read()
+
+
 def build_glue(force: bool = False) -> str:
-    header = os.path.join(ROOT, "include", "lory.h")
-    if not force and os.path.exists(GLUE) and all(os.path.getmtime(p) <= os.path.getmtime(GLUE) for p in (GLUE_SRC, header)):
+    if not force and glue_is_current():
         return GLUE
     import sysconfig
 
@@ -46,7 +64,7 @@ def build_glue(force: bool = False) -> str:
     libdir = os.path.join(os.path.dirname(torch.__file__), "lib")
     tmp = f"{GLUE}.{os.getpid()}"      # moved into place: another process may be importing the module
     cmd = ([os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", "-DTORCH_EXTENSION_NAME=_torch_glue",
-            f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}"] + ["-I" + p for p in inc] + [GLUE_SRC] +
+            f'-DLORY_GLUE_TAG="{glue_tag()}"', f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}"] + ["-I" + p for p in inc] + [GLUE_SRC] +
            ["-L" + libdir, "-Wl,-rpath," + libdir, "-ltorch", "-ltorch_cpu", "-ltorch_cuda", "-ltorch_python", "-lc10",
             "-lc10_cuda", "-ldl", "-o", tmp])
     res = subprocess.run(cmd, capture_output=True, text=True)

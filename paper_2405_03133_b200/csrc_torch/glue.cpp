@@ -220,6 +220,7 @@ Tensor decode(const Tensor& x_in, const Tensor& W1, const Tensor& W2, const Tens
 }  // namespace
 
 PYBIND11_MODULE(_torch_glue, m) {
+  m.attr("tag") = LORY_GLUE_TAG;
   m.def("bind", &bind);
   m.def("moe", &moe);
   m.def("forward", &forward);

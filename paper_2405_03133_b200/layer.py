@@ -26,7 +26,7 @@ _lock = threading.Lock()
 
 def _glue():
     """The C++ side of this file (autograd nodes, allocations, argument marshalling): loaded by the first call that needs it,
-    and built before that if need be."""
+    and built before that if it is missing or its sources have changed."""
     if _module is None:
         _load()
     return _module
@@ -37,11 +37,12 @@ def _load():
     with _lock:
         if _module is not None:
             return
+        from . import build
         _lory.load()
+        build.build_glue()
         try:
             glue = importlib.import_module("._torch_glue", __package__)
-        except ImportError:
-            from . import build
+        except ImportError:     # built for another interpreter
             build.build_glue(force=True)
             glue = importlib.import_module("._torch_glue", __package__)
         glue.bind(_lory.LIB_PATH, _lory._check)
