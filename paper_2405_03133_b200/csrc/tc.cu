@@ -634,14 +634,23 @@ static int launch_decode_mma(const lory_dims& D, const bf16* wa, const bf16* wb,
   return launch_overlapped(decode_mma_kernel<GATE>, dim3((unsigned)(tiles < sm_count() ? tiles : sm_count())), 224,
                            p.stages * stage + p.tail + 1024, st, 1, m_w, m_w3, m_x, p);
 }
-static bool decode_supported(const lory_dims& D) { return (D.flags & LORY_FLAG_REUSE_MERGED) && D.T <= 64; }
+// Where the decode kernels below beat the grouped GEMMs: up to 64 tokens, but with d <= 512, where a tile is a few stages and all
+// start and end, past 32 tokens only while there is at most a gate tile per SM, past 16 while there are at most three.
+// us a call, decode kernels | grouped GEMMs: 64 tokens, d = 256, f = 688: 12 sequences 14.5 | 16.4, 16: 19.0 | 16.0, 32: 24.3 |
+// 18.5; d = 512, f = 1376, 32: 44.8 | 38.9; 32 tokens: 16: 24.5 | 22.6, 24: 37.9 | 29.2, 64: 93 | 59; 17 tokens, d = 448, f = 1200, 16:
+// 18.7 | 20.5, 24: 26.0 | 22.6, 64: 74 | 48.  Wider, 64 tokens: d = 640, f = 1728, 32: 56.5 | 54.1, d = 768, 48: 95.5 | 98.1.
+static long gate_tiles(const lory_dims& D) { return ceil_div(D.f, 64) * D.B * (D.L / D.T); }
+static bool decode_supported(const lory_dims& D) {
+  if (!(D.flags & LORY_FLAG_REUSE_MERGED) || D.T > 64) return false;
+  return D.d > 512 || D.T <= 16 || gate_tiles(D) <= (D.T > 32 ? 1L : 3L) * sm_count();
+}
 // Past 16 tokens decode_kernel fetches as many token as weight bytes, and decode_mma_kernel takes over where its larger tiles
 // keep the SMs busy: past 32 tokens from half a tile per SM on, below from one and a half, and only with d > 512 (a tile of
 // fewer than three stages is all start and end).  us a call, decode_kernel or grouped GEMM -> decode_mma_kernel: 48 tokens, 4
 // sequences, d = 2048: 76 -> 55; 40, 8, d = 1024: 47 -> 35; 64, 1, d = 2048: 38 -> 33; 24, 8, d = 1024: 40 -> 33; on the other side
 // of the line 20, 1, d = 1024: 12 -> 19; 24, 2, d = 2048: 34 -> 39; 17, 32, d = 256: 16.5 -> 19.4.
 static bool decode_on_mma(const lory_dims& D) {
-  const long tiles = ceil_div(D.f, 64) * D.B * (D.L / D.T);
+  const long tiles = gate_tiles(D);
   return D.T > 32 ? 2 * tiles >= sm_count() : D.T > 16 && D.d > 512 && 2 * tiles >= 3L * sm_count();
 }
 // (the debug build's bounds checks may report before a block of the same kernel has cleared the word)
