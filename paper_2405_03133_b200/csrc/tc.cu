@@ -18,6 +18,7 @@
 
 #include "decode_tc.cuh"
 #include "gemm_tc.cuh"
+#include "merge_tc.cuh"
 #include "stage2_tc.cuh"
 #include "stream_tc.cuh"
 #include "wgrad_tc.cuh"
@@ -432,6 +433,48 @@ static int check_vector_aligned(const void* const* ptrs, int n) {
   return LORY_OK;
 }
 
+// Where the merge runs on tcgen05 (merge_tc.cuh), because the streaming kernel's matrix instructions would take longer than its
+// bytes.  us, streaming | tcgen05, d = 1024, f = 2752: E = 56: S = 96: 516 | 434, 128: 634 | 625, 192: 939 | 847, 256: 1322 | 976, 320:
+// 1657 | 1568, 512: 3159 | 2253; E = 48: 192: 741 | 764, 224: 903 | 859, 256: 1082 | 1048, 320: 1301 | 1471, 512: 2282 | 2185;
+// E = 32: 256: 851 | 1000.  (A tcgen05 launch has up to 256 segments and reads all experts: 320 segments cost it two.)
+static bool merge_on_tcgen05(const lory_dims& D) {
+  const int S = D.B * (D.L / D.T);
+  return D.E > 48 ? S > 64 : D.E > 32 && ((S > 192 && S <= 256) || S > 384);
+}
+static int launch_merge_tcgen05(const lory_dims& D, const WsPtrs& q, const bf16* const src[3], bf16* const dst[3],
+                                cudaStream_t st) {
+  const int S = D.B * (D.L / D.T), Ep = e_pad(D);
+  const int R[3] = {D.f, D.f, D.d}, C[3] = {D.d, D.d, D.f};
+  MergeMaps maps;
+  MergeParams p = {};
+  p.Epad16 = e_pad16(D); p.status = q.status;
+  LORY_TRY(make_map(&maps.w_hi, q.w_hi, Ep, S, 1, Ep, 0, 128));
+  LORY_TRY(make_map(&maps.w_lo, q.w_lo, Ep, S, 1, Ep, 0, 128));
+  int acc = 0;
+  for (int k = 0; k < 3; ++k) {
+    LORY_TRY(make_expert_map(&maps.theta[k], src[k], R[k], C[k], D.E, p.Epad16));
+    LORY_TRY(make_blocked_map(&maps.out[k], dst[k], R[k], C[k], S, 1, 32, 1, 1));
+    p.ctiles[k] = (C[k] + 63) / 64;
+    acc += (R[k] + 63) / 64 * 16 * p.ctiles[k];   // padded rows are written too (as zeros)
+    p.tile_end[k] = acc;
+  }
+  p.stage_bytes = 4 * p.Epad16 * 128;
+  const int S_launch = S < 256 ? S : 256;   // the routing weights of at most 256 segments stay in shared memory
+  const int fixed = (S_launch + 127) / 128 * 32768 + 32768 + 1024;   // weights, output staging
+  p.stages = (kMaxSmem - fixed) / p.stage_bytes;
+  if (p.stages > 8) p.stages = 8;
+  static bool attr_set[kMaxDevices];
+  LORY_TRY(allow_dynamic_smem(merge_kernel, kMaxSmem, attr_set));
+  const int grid = p.tile_end[2] < sm_count() ? p.tile_end[2] : sm_count();
+  for (int base = 0; base < S; base += 256) {
+    p.seg_base = base;
+    p.s_tiles = ((S - base < 256 ? S - base : 256) + 127) / 128;
+    ProfScope ps("merge", st);
+    LORY_TRY(launch_kernel(false, merge_kernel, dim3((unsigned)grid), 192, fixed + p.stages * p.stage_bytes, st, 1, maps, p));
+  }
+  return LORY_OK;
+}
+
 template <int KT, int U, int NW>
 static int launch_merge_t(const StreamMergeParams& p, cudaStream_t st) {
   ProfScope ps("merge", st);
@@ -442,6 +485,7 @@ static int launch_merge(const lory_dims& D, const WsPtrs& q, const bf16* const s
                         cudaStream_t st) {
   const int R[3] = {D.f, D.f, D.d}, C[3] = {D.d, D.d, D.f};
   LORY_TRY(check_vector_aligned((const void* const*)src, 3));
+  if (merge_on_tcgen05(D)) return launch_merge_tcgen05(D, q, src, dst, st);
   StreamMergeParams p = {};
   unsigned long pieces = 0;
   for (int k = 0; k < 3; ++k) {
