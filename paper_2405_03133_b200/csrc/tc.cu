@@ -371,21 +371,23 @@ size_t tc_adjoint_ring_elems(const lory_dims& D) {
 }
 
 // How a grouped GEMM is cut into tiles: the shape with the least (rounds over the GPU) x (time of a 64-deep step of a tile).
-// The step times are measured ones (us, d = 1024..2048, bf16); they grow far less than the tile does, because a step is a
-// chain of a load, a barrier and four MMAs, so the largest tiles win as long as they fill the GPU, and smaller ones where
-// they would leave SMs idle.  us, largest tile -> the one picked: gemm2 of 8 segments of 256 tokens, d = 1024, f = 2752:
-// 25 -> 23, dx 43 -> 39; gemm2 of 2 segments of 1000 tokens: 36 -> 23 (it used to run on 64-column tiles); 9 segments of
-// 200 tokens on CTA pairs: gemm1 24.9 -> 22.9.
+// The step times grow far less than the tile does, because a step is a chain of a load, a barrier and four MMAs, so the largest
+// tiles win as long as they fill the GPU, and smaller ones where they would leave SMs idle.  us a call, largest tile -> the one
+// picked: gemm2 of 8 segments of 256 tokens, d = 1024, f = 2752: 25 -> 23, dx 43 -> 39; gemm2 of 2 segments of 1000 tokens: 36 ->
+// 23 (it used to run on 64-column tiles); 9 segments of 200 tokens on CTA pairs: gemm1 24.9 -> 22.9.
+// The table's times (us, d = 1024..2048) are from before the issuing threads were elected (ptx::elect_one) and serve as ratios.
+// With them: gemm2, d = 1024, one group out of L2 | a group per 256 or 128 rows: pair 256 columns 0.34 | 0.52, 256: 0.52 | 0.83, 128:
+// 0.20 | 0.46, 64: 0.20 | 0.27.
 struct TileShape {
-  bool pair;  // 256-row tiles on CTA pairs, else 128-row tiles
+  bool pair;  // 256-row tiles on CTA pairs (256 columns), else 128-row tiles
   int bn;     // columns (of both products together for the gate / up projections)
 };
 static TileShape pick_tiles(int M, int N, int groups, bool narrow) {
-  static const struct { TileShape t; double step; } shapes[5] = {
-      {{true, 256}, 0.47}, {{false, 256}, 0.54}, {{true, 128}, 0.42}, {{false, 128}, 0.40}, {{false, 64}, 0.36}};
+  static const struct { TileShape t; double step; } shapes[4] = {
+      {{true, 256}, 0.47}, {{false, 256}, 0.54}, {{false, 128}, 0.40}, {{false, 64}, 0.36}};
   TileShape best = {false, 256};
   double least = 1e30;
-  for (int i = 0; i < (narrow ? 5 : 2); ++i) {
+  for (int i = 0; i < (narrow ? 4 : 2); ++i) {
     const TileShape t = shapes[i].t;
     const long tiles = ceil_div(M, t.pair ? 256 : 128) * ceil_div(N, t.bn) * groups;
     const double cost = (double)ceil_div(tiles, sm_count() / (t.pair ? 2 : 1)) * shapes[i].step;
@@ -773,14 +775,12 @@ int tc_ffn_forward(const lory_dims& D, const Layout& Lo, char* ws, const bf16* x
     p.residual = residual;   // y = residual + H Wbar2^T: the block's skip connection rides in the epilogue
     auto go = [&](auto launch) { return launch("gemm2", m_h, m_h, m_b2, m_b2, m_y, m_y, m_y, p, st, nullptr, nullptr); };
     if (residual) {
-      if (ts.pair && ts.bn == 256) LORY_TRY(go(launch_tc<false, false, 256, MODE_PLAIN, EPI_BF16_RESADD, true, false, 2>));
-      else if (ts.pair) LORY_TRY(go(launch_tc<false, false, 128, MODE_PLAIN, EPI_BF16_RESADD, true, false, 2>));
+      if (ts.pair) LORY_TRY(go(launch_tc<false, false, 256, MODE_PLAIN, EPI_BF16_RESADD, true, false, 2>));
       else if (ts.bn == 256) LORY_TRY(go(launch_tc<false, false, 256, MODE_PLAIN, EPI_BF16_RESADD, true>));
       else if (ts.bn == 128) LORY_TRY(go(launch_tc<false, false, 128, MODE_PLAIN, EPI_BF16_RESADD, true>));
       else LORY_TRY(go(launch_tc<false, false, 64, MODE_PLAIN, EPI_BF16_RESADD, true>));
     } else {
-      if (ts.pair && ts.bn == 256) LORY_TRY(go(launch_tc<false, false, 256, MODE_PLAIN, EPI_BF16, true, false, 2>));
-      else if (ts.pair) LORY_TRY(go(launch_tc<false, false, 128, MODE_PLAIN, EPI_BF16, true, false, 2>));
+      if (ts.pair) LORY_TRY(go(launch_tc<false, false, 256, MODE_PLAIN, EPI_BF16, true, false, 2>));
       else if (ts.bn == 256) LORY_TRY(go(launch_tc<false, false, 256, MODE_PLAIN, EPI_BF16, true>));
       else if (ts.bn == 128) LORY_TRY(go(launch_tc<false, false, 128, MODE_PLAIN, EPI_BF16, true>));
       else LORY_TRY(go(launch_tc<false, false, 64, MODE_PLAIN, EPI_BF16, true>));
@@ -844,8 +844,7 @@ int tc_ffn_backward(const lory_dims& D, const Layout& Lo, char* ws, const bf16* 
     TcGemmParams p = {};
     p.M = T; p.N = f; p.K = d; p.groups = S; p.status = q.status;
     auto go = [&](auto launch) { return launch("dh_dswiglu", m_dy, m_dy, m_b2, m_b2, m_dgo, m_duo, m_duo, p, st, &m_gi, &m_ui); };
-    if (ts.pair && ts.bn == 256) LORY_TRY(go(launch_tc<false, true, 256, MODE_PLAIN, EPI_DSWIGLU, true, false, 2>));
-    else if (ts.pair) LORY_TRY(go(launch_tc<false, true, 128, MODE_PLAIN, EPI_DSWIGLU, true, false, 2>));
+    if (ts.pair) LORY_TRY(go(launch_tc<false, true, 256, MODE_PLAIN, EPI_DSWIGLU, true, false, 2>));
     else if (ts.bn == 256) LORY_TRY(go(launch_tc<false, true, 256, MODE_PLAIN, EPI_DSWIGLU, true>));
     else if (ts.bn == 128) LORY_TRY(go(launch_tc<false, true, 128, MODE_PLAIN, EPI_DSWIGLU, true>));
     else LORY_TRY(go(launch_tc<false, true, 64, MODE_PLAIN, EPI_DSWIGLU, true>));
@@ -894,8 +893,7 @@ int tc_ffn_backward_dx(const lory_dims& D, const Layout& Lo, char* ws, const flo
   p.M = T; p.N = d; p.K = f; p.groups = S; p.status = q.status;
   p.rowvec = dh_bar; p.row_scale = 1.0f / (float)T;
   auto go = [&](auto launch) { return launch("dx", m_dg, m_du, m_b1, m_b3, m_dx, m_dx, m_dx, p, st, nullptr, nullptr); };
-  if (ts.pair && ts.bn == 256) return go(launch_tc<false, true, 256, MODE_DUALK, EPI_BF16_ROWADD, true, false, 2>);
-  if (ts.pair) return go(launch_tc<false, true, 128, MODE_DUALK, EPI_BF16_ROWADD, true, false, 2>);
+  if (ts.pair) return go(launch_tc<false, true, 256, MODE_DUALK, EPI_BF16_ROWADD, true, false, 2>);
   if (ts.bn == 256) return go(launch_tc<false, true, 256, MODE_DUALK, EPI_BF16_ROWADD, true>);
   if (ts.bn == 128) return go(launch_tc<false, true, 128, MODE_DUALK, EPI_BF16_ROWADD, true>);
   return go(launch_tc<false, true, 64, MODE_DUALK, EPI_BF16_ROWADD, true>);
