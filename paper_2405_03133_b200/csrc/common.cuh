@@ -60,7 +60,10 @@ struct ProfScope {
 // A kernel launched that way may have its CTAs on the GPU before the kernel in front of it has ended, so
 // that its own set-up (barriers, TMEM, descriptors) and the launch itself cost nothing.  EVERY CTA of such a kernel calls
 // pdl_wait() before it touches global memory: the call returns once the kernel in front has ended and its writes are
-// visible (and so, as that one waited too, everything before it).  pdl_launch() lets the next kernel's CTAs in; it takes
+// visible (and so, as that one waited too, everything before it).  One exception: the down projection of a decode call fetches
+// weights before it waits.  It may, because the gate kernel is the launch right in front of it, writes no weights, and lets
+// it in (pdl_launch) only after its own wait: whatever wrote the weights has ended by then.  A kernel placed between or in
+// front of those two has to keep that.  pdl_launch() lets the next kernel's CTAs in; it takes
 // effect when all CTAs of the grid have called it or ended, so they never take the place of a CTA that still has to start.
 // Not for a kernel whose split of an SM's memory into L1 and shared memory differs from its predecessor's in a way that
 // matters to it: an SM changes the split only when it is empty, so an overlapped kernel runs with the one it finds

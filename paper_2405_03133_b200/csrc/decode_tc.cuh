@@ -15,7 +15,7 @@
 // row).  The second kernel is launched while the first runs (programmatic dependent launch) and has its first weights on
 // the way before it waits for H.
 // us per call, grouped GEMM -> here, d = 1024, f = 2752, one token: 1 sequence 32.8 -> 9.0, 8: 45.5 -> 26.3, 32: 122 -> 85
-// (6.4 TB/s); 40 tokens, 4 sequences: 36.3 -> 30.5.
+// (6.4 TB/s).
 #pragma once
 #include <cuda.h>
 

@@ -337,8 +337,8 @@ __global__ void __launch_bounds__(128 * KG, 3) fma_gemm_kernel(const __grid_cons
 // The same for fp32 operands and too few tiles to fill the GPU: 32 x 64 tiles whose contraction is shared by the eight warps
 // of a CTA, each with a cp.async ring of its own (transposing on the way where the contraction runs along the stored rows)
 // and no barrier until the end, where the warps' sums meet in shared memory and every warp finishes one row in eight.  A lane
-// computes 8 x 8 outputs, which needs a quarter of the shared-memory reads per FMA of the 2 x 8 above.  us, before -> after,
-// 8 segments of 128 tokens, d = 256, f = 688: gemm2 31 -> 27, dx 49 -> 33.
+// computes 8 x 8 outputs, which needs a quarter of the shared-memory reads per FMA of the 2 x 8 above.  us, the kernel above ->
+// this one, 8 segments of 128 tokens, d = 256, f = 688: gemm2 31 -> 23, dx 53 -> 27.
 // -----------------------------------------------------------------------------------------------------------------
 struct Fma32 {
   static constexpr int KG = 8, BM = 32, BN = 64, BK = 16, STG = 3;

@@ -138,7 +138,7 @@ static int launch_fma32(const FmaArgs& a, long tiles, cudaStream_t st) {
 }
 
 // Tile choice.  128-row tiles have the best ratio of FMAs to shared-memory reads and need enough of them; below two per
-// SM 64-row tiles, below one per SM 32-row tiles (d = 256, f = 688, 8 segments of 128: dx 109, 60 and 44 us).  Two k-groups
+// SM 64-row tiles, below one per SM 32-row tiles (d = 256, f = 688, 8 segments of 128: dx 91, 62 and 54 us).  Two k-groups
 // per CTA where an SM gets fewer than three CTAs, and always with 32 rows, where a thread has too few FMAs between its
 // shared-memory reads to hide them (16-token segments, d = 301: 168 -> 136 us).  fp32 with less than half a 64-row tile per
 // SM: the kernel that shares a 32-row tile's contraction between eight warps.

@@ -88,7 +88,7 @@ stage2_kernel(const __grid_constant__ Stage2Maps maps, const Stage2Params p) {
   const int warp = ptx::warp_index(), lane = threadIdx.x & 31;
   const int num_tiles = p.tile_end[2];
   const int STAGES = p.stages;
-  const int NCB = p.ncb;   // 64-column blocks per tile (2; 3 on the fast path with 33..64 segments)
+  const int NCB = p.ncb;   // 64-column blocks per tile (2; 3 on the fast path)
   // tile -> (matrix k, row r, first column c0)
   auto decode = [&](int tile, int& k, int& r, int& c0) {
     k = tile < p.tile_end[0] ? 0 : (tile < p.tile_end[1] ? 1 : 2);

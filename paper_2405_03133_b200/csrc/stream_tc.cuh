@@ -86,8 +86,9 @@ __device__ __forceinline__ void b_fragments(const uint4 (&v)[4], uint32_t (&b)[8
 
 // -----------------------------------------------------------------------------------------------------------
 // Merge: Wbar_k[s, p] = sum_e w[s, e] W_k[e, p] into the blocked layout, A = (w_hi + w_lo), B = the experts, for any
-// number of segments.  KT = ceil(E / 16).  A warp loads U consecutive pieces of all experts into registers and then
-// walks the segments, 16 at a time, with the weight fragments the routing step has prepared (they stay in L1).
+// number of segments (with many of both the matrix instructions become the bound, and merge_tc.cuh takes over).
+// KT = ceil(E / 16).  A warp loads U consecutive pieces of all experts into registers and then walks the segments, 16 at a
+// time, with the weight fragments the routing step has prepared (they stay in L1).
 // HBM-bound: algorithmic bytes 2 (E + S) per parameter.  The CTAs are small (two warps) and each does its pieces and
 // ends, so the hardware hands out work as SMs get through theirs: SMs differ by 1.4 x in the rate at which they get
 // writes out, and every persistent grid (the tcgen05 kernel this one replaced among them) waits for the slowest.

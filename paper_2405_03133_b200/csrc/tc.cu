@@ -166,9 +166,10 @@ static int launch_tc(const char* label, const CUtensorMap& a0, const CUtensorMap
 }
 
 // One per-segment weight gradient C_g = A_g^T B_g (K = T): the resident-operand kernel for CTA-pair tiles with short
-// segments (its strips run along the dimension with more tiles), else the grouped GEMM.  Measured on one GPU
-// (d = 2048, f = 5504, E = 32; three launches): T = 64: 3.69 -> 3.53 ms, T = 128: 1.99 -> 1.82 ms; at T = 256 the two
-// kernels tie (d = 1024, f = 2752: 0.591 vs 0.600 ms; d = 2048: 1.14 vs 1.11 ms) and the grouped GEMM stays.
+// segments (its strips run along the dimension with more tiles), else the grouped GEMM.  ms, three launches, d = 2048, f = 5504,
+// grouped | resident: T = 64: 256 segments 11.33 | 10.77, 64: 2.60 | 2.55, 48: 2.05 | 2.30, 16: 0.68 | 0.70; T = 128: 128 segments
+// 6.47 | 5.87, 64: 2.93 | 2.82; d = 1024, f = 2752, T = 64: 256: 2.63 | 2.67, 64: 0.67 | 0.73: the line serves the case with the most
+// weights and costs up to a tenth with few segments.  At T = 256 the two tie (d = 1024: 0.591 | 0.600; d = 2048: 1.14 | 1.11).
 static int launch_wgrad(const CUtensorMap& a, const CUtensorMap& b, const CUtensorMap& c, int M, int N, int K, int groups,
                         bool pairs, uint32_t* status, cudaStream_t st) {
   if (pairs && K <= 128) {
@@ -275,9 +276,10 @@ static int stage2_grid(const lory_dims& D) {
 }
 
 // Where the adjoint of the merge runs as a streaming kernel (stream_tc.cuh): as long as a warp can keep the dw sums of
-// all segments and experts (and, for 17..32 experts, its pieces' rows in flight) beside its working set.  Measured at
-// d = 1024, f = 2752 against the tcgen05 kernel: E = 16, S = 64: 306 -> 271 us; E = 32, S = 48: 365 -> 326 us, but S = 64:
-// 381 -> 475 us; E = 48, S = 32: 617 -> 398 us.
+// all segments and experts (and, for 17..32 experts, its pieces' rows in flight) beside its working set.  us at
+// d = 1024, f = 2752, tcgen05 kernel | this one: E = 16: S = 16: 190 | 150, 64: 333 | 271; E = 32: S = 16: 285 | 250, 48: 365 | 325, 64:
+// 393 | 475; E = 48: S = 32: 517 | 397; E = 64: S = 16: 532 | 495, 32: 526 | 563 (d = 2048: 2390 | 2431).  Accumulating, d = 2048,
+// f = 5504, S = 16, two passes, one of them plain: E = 16: 2077 | 1291, E = 32: 3961 | 2544.
 static bool adjoint_streams(const lory_dims& D) {
   const int st = (D.B * (D.L / D.T) + 15) / 16, et = (D.E + 15) / 16;
   return st <= (et == 1 ? 4 : (et == 2 ? 3 : 2));
@@ -498,7 +500,8 @@ static int launch_merge(const lory_dims& D, const WsPtrs& q, const bf16* const s
   if (pieces > 0x7fffffffUL) return LORY_ERR_SHAPE;
   p.w_frag = (const uint4*)q.w_frag; p.S = D.B * (D.L / D.T); p.E = D.E;
   // Loads in flight per warp: 8 vectors per lane with up to 32 experts (two pieces of 16 experts or one of 32; two of 32
-  // cost occupancy: 1.13 instead of 1.02 ms at S = 64, d = 2048, f = 5504), one piece with more.
+  // cost occupancy: 1.13 instead of 1.02 ms at S = 64, d = 2048, f = 5504), one piece with more (past 48 experts two and four
+  // warps per CTA measure the same).
   switch ((D.E + 15) / 16) {
     case 1: return launch_merge_t<1, 2, 2>(p, st);
     case 2: return launch_merge_t<2, 1, 2>(p, st);
