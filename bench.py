@@ -127,9 +127,9 @@ def implementation_bytes_per_step(wl):
 # the digest of the CUDA sources at that time, and a different digest turns the reported traffic into null.
 NCU_TRAFFIC = {
     "C3": {
-        "sources_sha1": "cebe8cf3fc030c69f7acb3f3be5693b7b1ceb632",
-        "bytes": {"pool_router": 68e6, "merge": 2792e6, "gemm1_swiglu": 2017e6, "gemm2": 964e6, "dh_dswiglu": 1486e6,
-                  "wgrad": 908e6, "stage2": 3238e6, "router_backward": 3e6, "dx": 1875e6},
+        "sources_sha1": "8b5583b527a89cba626c37b4c63c3c19394f7642",
+        "bytes": {"pool_router": 68e6, "merge": 2643e6, "gemm1_swiglu": 2015e6, "gemm2": 965e6, "dh_dswiglu": 1490e6,
+                  "wgrad": 908e6, "stage2": 3535e6, "router_backward": 3e6, "dx": 1875e6},
     },
 }
 
