@@ -38,7 +38,7 @@ namespace lory {
 
 struct Stage2Maps {
   CUtensorMap w_hi, w_lo;  // (Epad, S, 1)   box (64, 128, 1); with E <= 32 both map the combined hi|lo table
-  CUtensorMap dwbar[3];    // blocked 5-D    box (64, 1, min(128, S rounded up to 8), 2, 1)
+  CUtensorMap dwbar[3];    // blocked 5-D    box (64, 1, min(128, S rounded up to 16), column blocks of a tile, 1)
   CUtensorMap theta[3];    // (C, E, R)      box (64, Epad16, 1)
   CUtensorMap out[3];      // (C, E, R)      box (64, 32, 1): one warp's 32 experts, rows clipped to E
 };
